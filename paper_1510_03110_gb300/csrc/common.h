@@ -32,6 +32,7 @@ struct LevelInst {
     long long gx;   // first global state index (N+1 states per instance)
     int N;          // horizon of this instance's problem at this level (0: instance absent)
     int top;        // 1 when this level is the instance's top level
+    int c0, c1;     // its chunks in the level's chunk list (filled when they are in instance order)
 };
 
 // Everything a tree kernel of one level reads and writes.  Matrices are
@@ -101,6 +102,12 @@ struct LevelArgs {
     int ext_batch;
 };
 
+// mhe_info (include/mhe.h), the layout the kernels write
+struct mhe_info_rec {
+    int status, level, chunk, stage, refine_iters, pad;
+    double relres, est_relerr;
+};
+
 // Residual kernel arguments (level 0).  Reads the caller's FP64 problem and
 // the FP64 iterate; writes the correction right-hand side in the compute type
 // of the tree (TR = double or float).
@@ -128,6 +135,28 @@ struct ResidArgs {
     // when set the residual's stage products run in double-float arithmetic on the
     // FP32 pipes, and only the vectors are read in FP64
     const float *Ahi, *Alo, *Bhi, *Blo, *Chi, *Clo, *Rhi, *Rlo;
+};
+
+// One solve with stored factors and its refinement as a single launch (solve.cuh):
+// a cluster of CTAs per instance walks every level's chunks of that instance.
+constexpr int kSolveLevels = 12;   // levels a fused solve takes (its arguments are kernel parameters)
+template <typename T>
+struct SolveArgs {
+    int batch, nlev;
+    int cluster;                       // CTAs per instance
+    int fused_rhs;                     // the factorisation ran the vector part: start with the down pass
+    int max_refine;
+    double tol;
+    // per level: the pass with the problem's right-hand side, and the corrections' pass
+    // (at index k and at index kSolveLevels + k)
+    LevelArgs<T> lv[2 * kSolveLevels];
+    ResidArgs<T> r;
+    const unsigned int* kinf;
+    unsigned int* dznorm;
+    int *iters, *active;
+    mhe_info_rec* info;
+    // the FP64 solution of the mixed precisions is accumulated: zeroed first (nullptr: not)
+    double *zx, *zw, *zl;
 };
 
 // MHE data (Eq. org_mhe, Section II) -> the FP32 working copies of the UFTOC

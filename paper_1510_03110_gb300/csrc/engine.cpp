@@ -194,6 +194,7 @@ int Engine::init(const mhe_dims& d, const ShapeOps* o, const Runtime* r, void* s
 
 int Engine::upload_plan()
 {
+    ordered = index_chunks(plan);
     // every host array of the plan with its device destination
     struct Piece {
         void* dst;
@@ -604,7 +605,7 @@ void Engine::narrow_solution()
 }
 
 template <typename T>
-void Engine::residual(const mhe_rhs* rhs, const double* x, const double* w, const double* lam, const int* act)
+ResidArgs<T> Engine::resid_args(const mhe_rhs* rhs, const double* x, const double* w, const double* lam) const
 {
     ResidArgs<T> r;
     memset(&r, 0, sizeof(r));
@@ -620,13 +621,20 @@ void Engine::residual(const mhe_rhs* rhs, const double* x, const double* w, cons
     r.rl = static_cast<T*>(rl); r.ra = static_cast<T*>(ra); r.rl0 = static_cast<T*>(rl0);
     r.ra0 = static_cast<T*>(ra0); r.rlN = static_cast<T*>(rlN); r.rx0 = static_cast<T*>(rx0);
     r.norms = norms;
-    r.active = act;
-    r.any_active = act ? any_mask : nullptr;
     r.C = mheC;
     r.R = mheR;
     if (mheC && sizeof(T) == 4 && rAh) {   // the double-float residual of the MHE form
         r.Ahi = rAh; r.Alo = rAl; r.Bhi = rBh; r.Blo = rBl; r.Chi = rCh; r.Clo = rCl; r.Rhi = rRh; r.Rlo = rRl;
     }
+    return r;
+}
+
+template <typename T>
+void Engine::residual(const mhe_rhs* rhs, const double* x, const double* w, const double* lam, const int* act)
+{
+    ResidArgs<T> r = resid_args<T>(rhs, x, w, lam);
+    r.active = act;
+    r.any_active = act ? any_mask : nullptr;
     rt->memset0(norms, sizeof(unsigned long long) * 3 * plan.batch, stream);
     mark(PH_RESID, 0, 1);
     launches += r.nstages > 0;
@@ -652,12 +660,91 @@ void Engine::convert_rhs(const mhe_rhs* rhs)
 }
 
 template <typename T>
+LevelArgs<T> Engine::vec_args(int k, const T* l, const T* a, const T* l0, const T* a0, const T* lN, const T* x0,
+                              const long long* off, T* x, T* w, T* lam, double* zx, double* zw, double* zl) const
+{
+    LevelArgs<T> g = args<T>(k);
+    g.rhs_off = off;
+    g.A = static_cast<const T*>(mA); g.B = static_cast<const T*>(mB);
+    g.Q = static_cast<const T*>(mQ); g.P0inv = static_cast<const T*>(mP0);
+    g.l = l; g.a = a; g.l0 = l0; g.a0 = a0; g.lN = lN;
+    g.x0 = x0;
+    if (k == 0) {
+        g.xd = x; g.wd = w; g.ld = lam;
+        g.zx = zx; g.zw = zw; g.zl = zl;
+        g.dznorm = zx ? dznorm : nullptr;
+    }
+    return g;
+}
+
+namespace {
+void launch_solve(const ShapeOps* ops, const SolveArgs<double>& p, void* s) { ops->solve64(p, s); }
+void launch_solve(const ShapeOps* ops, const SolveArgs<float>& p, void* s)
+{
+    if (p.r.C) ops->solve_mhe32(p, s);
+    else ops->solve32(p, s);
+}
+}  // namespace
+
+// A batch of few or small instances is bound by launches and by the latency of the small upper
+// levels: one launch takes the vector pass, the down pass and every correction of an instance in
+// a cluster of its own, which stops when the instance has converged.  Timing marks want a launch
+// per level pass; FP64 master levels, the literal down pass and the FP64-instruction MHE residual
+// have no fused form.
+template <typename T>
+bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
+                         bool fused)
+{
+    const bool fp64 = sizeof(T) == 8;
+    const size_t L = lv.size();
+    if (!ops->solve_cluster || !ordered || m64 || literal || mark_user || L > (size_t)kSolveLevels) return false;
+    if (mheC && (fp64 || !rAh)) return false;
+    if (fp64 ? !ops->solve64 : (mheC ? !ops->solve_mhe32 : !ops->solve32)) return false;
+    const int cl = ops->solve_cluster(fp64, plan.batch, plan.max_N);
+    if (cl < 1) return false;
+    SolveArgs<T> p;
+    memset(&p, 0, sizeof(p));
+    p.batch = plan.batch;
+    p.nlev = (int)L;
+    p.cluster = cl;
+    p.fused_rhs = fused;
+    p.max_refine = max_refine;
+    p.tol = tol;
+    T* d[3] = {static_cast<T*>(dx), static_cast<T*>(dw), static_cast<T*>(dl)};
+    for (int k = 0; k < (int)L; ++k) {
+        if (fp64)
+            p.lv[k] = vec_args<T>(k, l, a, nullptr, nullptr, nullptr, x0, in_off, reinterpret_cast<T*>(x),
+                                     reinterpret_cast<T*>(w), reinterpret_cast<T*>(lam), nullptr, nullptr, nullptr);
+        else
+            p.lv[k] = vec_args<T>(k, l, a, nullptr, nullptr, nullptr, x0, in_off, d[0], d[1], d[2], x, w, lam);
+        p.lv[kSolveLevels + k] = vec_args<T>(k, static_cast<const T*>(rl), static_cast<const T*>(ra), static_cast<const T*>(rl0),
+                                static_cast<const T*>(ra0), static_cast<const T*>(rlN), static_cast<const T*>(rx0),
+                                cmp_off, d[0], d[1], d[2], x, w, lam);
+    }
+    p.r = resid_args<T>(rhs, x, w, lam);
+    p.kinf = kinf;
+    p.dznorm = dznorm;
+    p.iters = iters;
+    p.active = active;
+    p.info = reinterpret_cast<mhe_info_rec*>(info_dev);
+    if (!fp64) { p.zx = x; p.zw = w; p.zl = lam; }
+    ++launches;
+    launch_solve(ops, p, stream);
+    return true;
+}
+
+template <typename T>
 int Engine::run_solve(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
                       mhe_info* info, bool fused)
 {
     const bool fp64 = sizeof(T) == 8;
     active_mask = nullptr;
     x0_hi = rhs->x0;   // FP64 master levels: the top chunks above level 0 read x~0 in FP64
+    if (solve_fused<T>(rhs, l, a, x0, x, w, lam, fused)) {
+        if (info) rt->copy(info, info_dev, sizeof(mhe_info) * plan.batch, stream);
+        if (rt->error() != 0) { err = "CUDA error during the solve"; return MHE_E_CUDA; }
+        return MHE_OK;
+    }
     if (!fused) pass_rhs<T>(l, a, nullptr, nullptr, nullptr);
     if (fp64) {
         pass_down<T>(l, a, nullptr, nullptr, x0, nullptr, reinterpret_cast<T*>(x), reinterpret_cast<T*>(w),

@@ -43,6 +43,14 @@ struct ShapeOps {
     long long gws64;
     int gws_teams;
     int team;   // lanes per subproblem team of these kernels
+    // a whole solve with its refinement in one launch (solve.cuh), or nullptr: FP64, FP32
+    // with the Q-form residual, FP32 with the double-float MHE-form residual
+    void (*solve64)(const SolveArgs<double>&, void* stream);
+    void (*solve32)(const SolveArgs<float>&, void* stream);
+    void (*solve_mhe32)(const SolveArgs<float>&, void* stream);
+    // CTAs per instance that solve takes for a batch whose longest horizon is max_N;
+    // 0: one launch per level pass is the faster way
+    int (*solve_cluster)(int fp64, int batch, int max_N);
 };
 
 // Everything one compiled shape provides (one entry per shape and team width).
@@ -178,6 +186,7 @@ public:
     void* upload_stage = nullptr;
     size_t upload_stage_bytes = 0;
     size_t upload_need = 0;
+    bool ordered = false;               // every level's chunks are in instance order
     bool factored = false;
     std::string err;
 
@@ -232,6 +241,16 @@ private:
     int run_solve(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
                   mhe_info* info, bool skip_first_rhs);
     int upload_plan();
+    // the arguments of one level's vector passes for the right-hand side (l, a, ..., x0)
+    template <typename T>
+    LevelArgs<T> vec_args(int k, const T* l, const T* a, const T* l0, const T* a0, const T* lN, const T* x0,
+                          const long long* off, T* x, T* w, T* lam, double* zx, double* zw, double* zl) const;
+    // the solve and its refinement in one launch, when the shape and the batch suit it
+    template <typename T>
+    bool solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
+                     bool fused);
+    template <typename T>
+    ResidArgs<T> resid_args(const mhe_rhs* rhs, const double* x, const double* w, const double* lam) const;
     template <typename T>
     void residual(const mhe_rhs* rhs, const double* x, const double* w, const double* lam, const int* act);
     template <typename T>

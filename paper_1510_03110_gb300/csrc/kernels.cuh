@@ -9,6 +9,7 @@
 
 #include "engine.h"
 #include "resid.cuh"
+#include "solve.cuh"
 #include "tree.cuh"
 
 namespace mhe {
@@ -23,14 +24,15 @@ enum { OP_REDUCE = 0, OP_RHS = 1, OP_DOWN = 2, OP_REDUCE_TC = 3, OP_REDUCE_BF = 
 // the mbarrier and the TMEM address
 constexpr int kTcExtra = 8192 + 4;
 
-// shared-memory workspace (elements of T) one warp of a pass needs
-template <typename T, int NX, int OP>
+// shared-memory workspace (elements of T) one team of a pass needs
+template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int op_count()
 {
     return (OP == OP_REDUCE || OP == OP_DOWN_LIT)
                ? Ws<T, NX>::count
-               : (OP == OP_RHS ? Ws<T, NX>::count_rhs
-                               : (OP == OP_DOWN ? Ws<T, NX>::count_vec : Ws<T, NX>::count + kTcExtra));   // both tensor-core reductions
+               : (OP == OP_RHS ? VecWs<T, NX, NW, UPPER != 0>::rhs_count
+                               : (OP == OP_DOWN ? VecWs<T, NX, NW, UPPER != 0>::down_count
+                                                : Ws<T, NX>::count + kTcExtra));   // both tensor-core reductions
 }
 
 // CTAs of the residual kernel per SM its register budget is sized for
@@ -44,22 +46,29 @@ constexpr int kMaxTeams = 256 / MHE_TEAM;
 // shared memory the level kernels give their teams' workspaces per CTA
 constexpr int kLevelSmem = 224 * 1024;
 
-// teams per CTA: as many per-team workspaces as fit in kLevelSmem, at most kMaxTeams
-template <typename T, int NX, int OP>
+// the vector passes run in CTAs of 128 threads (one team, when it is wider): their workspaces are
+// rings of stage slots, and small CTAs fill an SM's shared memory closely
+template <int OP>
+constexpr bool vector_op() { return OP == OP_RHS || OP == OP_DOWN; }
+template <int OP>
+constexpr int op_max_teams()
+{
+    return vector_op<OP>() ? (MHE_TEAM >= 128 ? 1 : 128 / MHE_TEAM) : kMaxTeams;
+}
+
+// teams per CTA: as many per-team workspaces as fit in kLevelSmem, at most the op's
+template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int level_warps()
 {
-    return (kLevelSmem) / (int)(op_count<T, NX, OP>() * sizeof(T)) >= kMaxTeams
-               ? kMaxTeams
-               : ((kLevelSmem) / (int)(op_count<T, NX, OP>() * sizeof(T)) < 1
-                      ? 1
-                      : (kLevelSmem) / (int)(op_count<T, NX, OP>() * sizeof(T)));
+    constexpr int fit = kLevelSmem / (int)(op_count<T, NX, NW, UPPER, OP>() * sizeof(T));
+    return fit >= op_max_teams<OP>() ? op_max_teams<OP>() : (fit < 1 ? 1 : fit);
 }
 
 // a workspace the shared memory of one SM can hold (227 KB per CTA)
-template <typename T, int NX, int OP>
+template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr bool level_fits()
 {
-    return (long long)op_count<T, NX, OP>() * (long long)sizeof(T) <= 227LL * 1024;
+    return (long long)op_count<T, NX, NW, UPPER, OP>() * (long long)sizeof(T) <= 227LL * 1024;
 }
 
 // CTAs of 256 threads per SM the register allocation is sized for: the small
@@ -70,9 +79,15 @@ constexpr bool level_fits()
 // the right-hand-side pass, whose loads are unrolled wider, loses);
 // the n = 64 passes (one four-warp team per subproblem, a few hundred teams)
 // all take 255.
-template <typename T, int NX, int OP>
+template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int level_min_blocks()
 {
+    if (vector_op<OP>()) {
+        // as many CTAs as shared memory holds, with at least 64 registers a thread
+        constexpr int bytes = level_warps<T, NX, NW, UPPER, OP>() * op_count<T, NX, NW, UPPER, OP>() * (int)sizeof(T);
+        constexpr int fit = 228 * 1024 / (bytes + 1024);
+        return fit > 8 ? 8 : (fit < 1 ? 1 : fit);
+    }
     return NX >= 48 ? 1   // four-warp teams, a few per SM: every pass may take 255 registers
                     : (sizeof(T) == 4
                            ? (NX <= 8 ? 4
@@ -87,8 +102,8 @@ template <int NX, int NW>
 constexpr bool tc_shape()
 {
     return MHE_TEAM == 128 && NX % 16 == 0 && NW % 16 == 0 && NX + NW <= 128 && 2 * NX <= 128 &&
-           128 * NX * 4 <= 32 * 1024 && level_warps<float, NX, OP_REDUCE_TC>() == 1 &&
-           (long long)op_count<float, NX, OP_REDUCE_TC>() * 4 <= 227LL * 1024;
+           128 * NX * 4 <= 32 * 1024 && level_warps<float, NX, NW, 0, OP_REDUCE_TC>() == 1 &&
+           (long long)op_count<float, NX, NW, 0, OP_REDUCE_TC>() * 4 <= 227LL * 1024;
 }
 
 // Team slots of a global-memory workspace a context provides: two CTAs of one
@@ -98,18 +113,18 @@ constexpr bool tc_shape()
 constexpr int kGwsTeams = 2 * 152;
 
 template <typename T, int NX, int NW, int UPPER, int OP>
-__global__ void __launch_bounds__(256, level_min_blocks<T, NX, OP>()) k_level(LevelArgs<T> a)
+__global__ void __launch_bounds__(vector_op<OP>() ? 128 : 256, level_min_blocks<T, NX, NW, UPPER, OP>()) k_level(LevelArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int W = level_warps<T, NX, OP>();
-    if constexpr (!level_fits<T, NX, OP>()) {
+    constexpr int W = level_warps<T, NX, NW, UPPER, OP>();
+    if constexpr (!level_fits<T, NX, NW, UPPER, OP>()) {
         // the workspace of one subproblem exceeds an SM's shared memory (FP64 at
         // nx = 64): one team per CTA, its workspace in the CTA's slot of the
         // context's global workspace (L2-resident; the FP64 pipe, at about two
         // DFMAs per clock per SM, hides the L2 latency of the products)
         static_assert(W == 1 && (OP == OP_REDUCE || OP == OP_RHS || OP == OP_DOWN), "one CUDA-core team per CTA");
         if (a.any_active && *a.any_active == 0) return;
-        T* ws = a.gws + (size_t)blockIdx.x * op_count<T, NX, OP>();
+        T* ws = a.gws + (size_t)blockIdx.x * op_count<T, NX, NW, UPPER, OP>();
         for (int ci = blockIdx.x; ci < a.nchunks; ci += gridDim.x) {
             if (!chunk_in_bounds(a, ci)) continue;
             if constexpr (OP == OP_REDUCE) reduce_chunk<T, NX, NW, UPPER != 0>(a, ci, ws);
@@ -122,7 +137,7 @@ __global__ void __launch_bounds__(256, level_min_blocks<T, NX, OP>()) k_level(Le
     const int ci = blockIdx.x * W + team;
     if (ci >= a.nchunks) return;   // the whole team leaves together
     if (a.any_active && *a.any_active == 0) return;   // a refinement pass with every instance converged
-    T* sm = reinterpret_cast<T*>(smem_raw) + (size_t)team * op_count<T, NX, OP>();
+    T* sm = reinterpret_cast<T*>(smem_raw) + (size_t)team * op_count<T, NX, NW, UPPER, OP>();
     if constexpr (OP == OP_REDUCE_TC || OP == OP_REDUCE_BF) {
         // one team per CTA: TMEM (all 512 columns; one CTA fits an SM) and the mbarrier are the CTA's
         static_assert(W == 1 && sizeof(T) == 4, "one FP32 tensor-core team per CTA");
@@ -158,15 +173,15 @@ __global__ void __launch_bounds__(256, level_min_blocks<T, NX, OP>()) k_level(Le
 template <typename T, int NX, int NW, int UPPER, int OP>
 void launch_level_v(const LevelArgs<T>& a, void* stream)
 {
-    constexpr int W = level_warps<T, NX, OP>();
-    if constexpr (!level_fits<T, NX, OP>()) {
+    constexpr int W = level_warps<T, NX, NW, UPPER, OP>();
+    if constexpr (!level_fits<T, NX, NW, UPPER, OP>()) {
         // global-memory workspace: at most gws_teams CTAs of one team, no dynamic shared memory
         if (!a.gws || a.gws_teams < 1) return;   // the context holds no workspace slots: nothing is launched
         const int grid = a.nchunks < a.gws_teams ? a.nchunks : a.gws_teams;
         k_level<T, NX, NW, UPPER, OP><<<grid, MHE_TEAM, 0, (cudaStream_t)stream>>>(a);
         return;
     }
-    const size_t smem = (size_t)W * op_count<T, NX, OP>() * sizeof(T);
+    const size_t smem = (size_t)W * op_count<T, NX, NW, UPPER, OP>() * sizeof(T);
     static bool attr = false;
     if (!attr) {
         cudaFuncSetAttribute(k_level<T, NX, NW, UPPER, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -373,7 +388,7 @@ ShapeEntry make_shape()
     e.ops.nx = NX;
     e.ops.nw = NW;
     e.ops.team = MHE_TEAM;
-    if constexpr (level_fits<double, NX, OP_REDUCE>()) {
+    if constexpr (level_fits<double, NX, NW, 0, OP_REDUCE>()) {
         e.ops.reduce64 = &launch_level<double, NX, NW, OP_REDUCE>;
         e.ops.rhs64 = &launch_level<double, NX, NW, OP_RHS>;
         e.ops.down64 = &launch_level<double, NX, NW, OP_DOWN>;
@@ -394,7 +409,7 @@ ShapeEntry make_shape()
     e.ops.rhs32 = &launch_level<float, NX, NW, OP_RHS>;
     e.ops.down32 = &launch_level<float, NX, NW, OP_DOWN>;
     // the literal Algorithm 6 down pass, for the shapes whose reduction workspace fits an SM
-    if constexpr (level_fits<double, NX, OP_REDUCE>() && NX <= 32) {
+    if constexpr (level_fits<double, NX, NW, 0, OP_REDUCE>() && NX <= 32) {
         e.ops.down64lit = &launch_level<double, NX, NW, OP_DOWN_LIT>;
         e.ops.down32lit = &launch_level<float, NX, NW, OP_DOWN_LIT>;
     } else {
@@ -410,6 +425,16 @@ ShapeEntry make_shape()
     e.ops.resid_mhe32 = &launch_resid<NX, NW, float, NY>;
     e.ops.gws64 = 0;
     e.ops.gws_teams = 0;
+    if constexpr (NX <= 32) {
+        e.ops.solve64 = &launch_solve<double, NX, NW, 0>;
+        e.ops.solve32 = &launch_solve<float, NX, NW, 0>;
+        e.ops.solve_mhe32 = &launch_solve<float, NX, NW, NY>;
+        e.ops.solve_cluster = &solve_cluster<NX, NW, NY>;
+    } else {
+        e.ops.solve64 = nullptr;
+        e.ops.solve32 = e.ops.solve_mhe32 = nullptr;
+        e.ops.solve_cluster = nullptr;
+    }
     e.ny = NY;
     e.assemble = &launch_assemble<NX, NW, NY>;
     return e;
@@ -421,11 +446,11 @@ ShapeEntry make_shape()
 template <int NX, int NW>
 void set_fp64_global_ops(ShapeOps& o)
 {
-    static_assert(!level_fits<double, NX, OP_REDUCE>(), "shapes whose FP64 workspace fits use make_shape");
+    static_assert(!level_fits<double, NX, NW, 0, OP_REDUCE>(), "shapes whose FP64 workspace fits use make_shape");
     o.reduce64 = &launch_level<double, NX, NW, OP_REDUCE>;
     o.rhs64 = &launch_level<double, NX, NW, OP_RHS>;
     o.down64 = &launch_level<double, NX, NW, OP_DOWN>;
-    o.gws64 = op_count<double, NX, OP_REDUCE>();
+    o.gws64 = op_count<double, NX, NW, 0, OP_REDUCE>();
     o.gws_teams = kGwsTeams;
 }
 

@@ -98,7 +98,8 @@ struct Entry {
 template <int NX, int NW>
 Entry entry()
 {
-    return Entry{NX, NW, &k_serial_noalloc<NX, NW>, mhe::Ws<double, NX>::count * sizeof(double)};
+    constexpr int c = mhe::max_int(mhe::Ws<double, NX>::count, mhe::VecWs<double, NX, NW, false>::down_count);
+    return Entry{NX, NW, &k_serial_noalloc<NX, NW>, c * sizeof(double)};
 }
 
 const Entry kEntries[] = {entry<1, 1>(),   entry<2, 1>(),   entry<3, 2>(),    entry<4, 2>(),   entry<6, 3>(),

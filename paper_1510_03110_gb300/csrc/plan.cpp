@@ -54,7 +54,7 @@ int make_plan(int n, int m, const int* N, int batch, int leaf_len, int branching
         for (int k = 0;; ++k) {
             if ((int)plan.levels.size() <= k) {
                 plan.levels.emplace_back();
-                plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0});
+                plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0, 0, 0});
             }
             PlanLevel& L = plan.levels[k];
             LevelInst& li = L.li[b];
@@ -83,7 +83,7 @@ int make_plan(int n, int m, const int* N, int batch, int leaf_len, int branching
             // the next level exists for this instance; its bases are the current counters
             if ((int)plan.levels.size() <= k + 1) {
                 plan.levels.emplace_back();
-                plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0});
+                plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0, 0, 0});
             }
             PlanLevel& U = plan.levels[k + 1];
             PlanLevel& L2 = plan.levels[k];   // re-take: emplace_back may move
@@ -105,6 +105,21 @@ int make_plan(int n, int m, const int* N, int batch, int leaf_len, int branching
         }
     }
     return 0;
+}
+
+bool index_chunks(Plan& plan)
+{
+    for (PlanLevel& L : plan.levels) {
+        int prev = -1;
+        for (int i = 0; i < (int)L.chunks.size(); ++i) {
+            const int b = L.chunks[i].inst;
+            if (b < prev || b >= plan.batch) return false;
+            if (b != prev) L.li[b].c0 = i;
+            L.li[b].c1 = i + 1;
+            prev = b;
+        }
+    }
+    return true;
 }
 
 namespace {
@@ -179,7 +194,7 @@ int make_serve_plan(int n, int m, const std::vector<ServeWindow>& w, int leaf, i
     auto level = [&](int k) -> PlanLevel& {
         while ((int)plan.levels.size() <= k) {
             plan.levels.emplace_back();
-            plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0});
+            plan.levels.back().li.assign(batch, LevelInst{0, 0, 0, 0, 0, 0});
             dirty.emplace_back();
         }
         return plan.levels[k];

@@ -46,6 +46,9 @@ int make_plan(int n, int m, const int* N, int batch, int leaf_len, int branching
 // A plan whose leaf chunks may have a rank-deficient Q^_w: leaf_len * nw < nx.
 inline bool needs_rank_revealing(int n, int m, int leaf_len) { return (long long)leaf_len * m < n; }
 
+// c0, c1 of every level's instances; false when some level's chunks are not in instance order.
+bool index_chunks(Plan& plan);
+
 // Chunk bounds of a level problem of horizon Nk with chunk length L: all chunks
 // have length L except the last (1..L stages); at least two chunks.
 void chunk_bounds(int Nk, int L, std::vector<int>& bnd);

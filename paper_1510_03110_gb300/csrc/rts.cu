@@ -66,7 +66,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
         const double* P0i = r.P0inv + (long long)b * NX * NX;
         mhe::wcopy<NX * NX>([&](int idx) { return P0i[idx]; },
                             [&](int idx, T v) { s.G[idx % NX + (idx / NX) * ld] = v; });
-        bad |= mhe::chol_inplace<T, NX, NX>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NX, true>(s, s.G, 1e-14);
         auto id = [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); };
         auto getY = [&](int i, int c) -> T { return s.PB[i + c * ld]; };
         auto putY = [&](int i, int c, T v) { s.PB[i + c * ld] = v; };
@@ -101,7 +101,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
             });
         // V^{-1} -> s.H: Cholesky of V in s.G, then two solves against the identity
         mhe::wfor(NY * NY, [&](int idx) { s.G[idx % NY + (idx / NY) * ld] = s.V[idx % NY + (idx / NY) * ld]; });
-        bad |= mhe::chol_inplace<T, NX, NY>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NY, true>(s, s.G, 1e-14);
         {
             auto id = [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); };
             auto getY = [&](int i, int c) -> T { return s.Tt[i + c * ld]; };
@@ -124,7 +124,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
             for (int p = 0; p < NX; ++p) acc -= s.K[i + p * ld] * s.v[p];
             s.e[i] = acc;
         });
-        bad |= mhe::chol_inplace<T, NX, NY>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NY, true>(s, s.G, 1e-14);
         // Y = L_S^{-1} CP (s.Tt), y = L_S^{-1} innovation (s.tmp)
         {
             auto rhs = [&](int i, int c) -> T { return c < NX ? s.PB[i + c * ld] : s.e[i]; };
@@ -157,7 +157,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
         });
         // B W^{-1} B^T = Z^T Z with Z = L_W^{-1} B^T (NW x n, s.Tt)
         mhe::wfor(NW * NW, [&](int idx) { s.G[idx % NW + (idx / NW) * ld] = s.Qw[idx % NW + (idx / NW) * ld]; });
-        bad |= mhe::chol_inplace<T, NX, NW>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NW, true>(s, s.G, 1e-14);
         {
             auto rhs = [&](int i, int c) -> T { return B[c + i * NX]; };
             auto get = [&](int i, int c) -> T { return s.Tt[i + c * ld]; };
@@ -209,7 +209,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
         mhe::wcopy<NX * NX>([&](int idx) { return PP(k + 1)[idx]; },
                             [&](int idx, T v) { s.G[idx % NX + (idx / NX) * ld] = v; });
         mhe::wfor(NX, [&](int i) { s.e[i] = s.v[i] - XP(k + 1)[i]; });
-        bad |= mhe::chol_inplace<T, NX, NX>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NX, true>(s, s.G, 1e-14);
         {
             auto rhs = [&](int i, int) -> T { return s.e[i]; };
             auto gety = [&](int i, int) -> T { return s.tmp[i]; };
@@ -246,7 +246,7 @@ MHE_DEV void rts_instance(const RtsArgs& r, int b, double* smem)
         // ws_k = w~ + W^{-1} B^T u: Cholesky of W in s.G, two solves
         mhe::wcopy<NW * NW>([&](int idx) { return R[idx % NW + (idx / NW) * NR]; },
                             [&](int idx, T v) { s.G[idx % NW + (idx / NW) * ld] = v; });
-        bad |= mhe::chol_inplace<T, NX, NW>(s, s.G, 1e-14);
+        bad |= mhe::chol_inplace<T, NX, NW, true>(s, s.G, 1e-14);
         {
             auto rhs = [&](int i, int) -> T { return s.k[i]; };
             auto gety = [&](int i, int) -> T { return s.tmp[i]; };

@@ -30,25 +30,14 @@
 
 #include "common.h"
 #include "f32conv.h"
+#include "stage.cuh"
 #include "tc.cuh"
+#include "vec.cuh"
 #include "warp.cuh"
 #include "wgemm.cuh"
 
 namespace mhe {
 MHE_TEAM_NS_BEGIN
-
-enum { KIND_LEAF = 0, KIND_ARRIVAL = 1, KIND_UPPER = 2 };
-
-// Leading dimension of the workspace matrices: a multiple of the 16-byte
-// vector (V elements) so every column starts 16-byte aligned, with an odd
-// number of vectors per column so neighbouring columns start in different
-// bank groups.
-constexpr int pick_ld(int n, int v)
-{
-    int l = n;
-    while (l % v != 0 || (l / v) % 2 == 0) ++l;
-    return l;
-}
 
 // Shared-memory workspace of one team (every matrix slot holds up to NX x NX;
 // columns and vectors 16-byte aligned for the vector loads of wgemm_tn).
@@ -69,27 +58,6 @@ struct Ws {
         P = p; p += slot; V = p; p += slot; Qw = p; p += slot; A = p; p += slot;
         Tt = p; p += slot; B = p; p += slot; PB = p; p += slot; H = p; p += slot;
         K = p; p += slot; G = p; p += slot;
-        Psi = p; p += nv; v = p; p += nv; u = p; p += nv; e = p; p += nv;
-        tv = p; p += nv; g = p; p += nv; k = p; p += nv; tmp = p; p += nv;
-        sc = p;
-    }
-    // right-hand-side pass: only A, B, K, G and the vectors
-    static constexpr int count_rhs = (4 * slot + 8 * nv + 8 + VEC - 1) / VEC * VEC;
-    MHE_DEV void carve_rhs(T* base)
-    {
-        T* p = base;
-        P = V = Qw = Tt = PB = H = nullptr;
-        A = p; p += slot; B = p; p += slot; K = p; p += slot; G = p; p += slot;
-        Psi = p; p += nv; v = p; p += nv; u = p; p += nv; e = p; p += nv;
-        tv = p; p += nv; g = p; p += nv; k = p; p += nv; tmp = p; p += nv;
-        sc = p;
-    }
-    // down pass: the vectors only
-    static constexpr int count_vec = (8 * nv + 8 + VEC - 1) / VEC * VEC;
-    MHE_DEV void carve_vectors(T* base)
-    {
-        T* p = base;
-        P = V = Qw = A = Tt = B = PB = H = K = G = nullptr;
         Psi = p; p += nv; v = p; p += nv; u = p; p += nv; e = p; p += nv;
         tv = p; p += nv; g = p; p += nv; k = p; p += nv; tmp = p; p += nv;
         sc = p;
@@ -123,57 +91,6 @@ MHE_DEV void tri_ij(int idx, int& i, int& j)
     j = jj;
     i = idx - jj * (jj + 1) / 2;
 }
-
-// Data of one stage.  LEAF: the caller's stage arrays (Q is (n+m)^2).
-// ARRIVAL: A = B = I, Q = diag(0, P~0^{-1}).  UPPER: a master-problem stage in
-// square-root form: A = A^, B = R^T, Q = blkdiag(Q^_x, I), l = (l^_x, 0),
-// where R^T R = Q^_w is the Cholesky factorisation of the T-form Q^_w = B^.
-template <typename T>
-struct StageRef {
-    const T *A, *B, *Q, *Qx, *Qw0, *l, *a;
-};
-
-template <typename T, int KIND, int NX, int MT>
-struct Acc {
-    static MHE_DEV T A(const StageRef<T>& s, int i, int j)
-    {
-        return KIND == KIND_ARRIVAL ? (T)(i == j ? 1 : 0) : s.A[i + j * NX];
-    }
-    static MHE_DEV T B(const StageRef<T>& s, int i, int j)
-    {
-        return KIND == KIND_ARRIVAL ? (T)(i == j ? 1 : 0) : s.B[i + j * NX];
-    }
-    static MHE_DEV T qx(const StageRef<T>& s, int i, int j)
-    {
-        if (KIND == KIND_LEAF) return s.Q[i + j * (NX + MT)];
-        if (KIND == KIND_UPPER) return s.Qx[i + j * NX];
-        return (T)0;
-    }
-    static MHE_DEV T qxw(const StageRef<T>& s, int i, int j)
-    {
-        return KIND == KIND_LEAF ? s.Q[i + (NX + j) * (NX + MT)] : (T)0;
-    }
-    static MHE_DEV T qw(const StageRef<T>& s, int i, int j)
-    {
-        if (KIND == KIND_LEAF) return s.Q[(NX + i) + (NX + j) * (NX + MT)];
-        if (KIND == KIND_UPPER) return (T)(i == j ? 1 : 0);   // square-root master stage
-        return s.Qw0[i + j * NX];
-    }
-    // entry (i, j) of the stage Hessian [[Q_x, Q_xw], [Q_xw^T, Q_w]], i, j < n + m
-    static MHE_DEV T q(const StageRef<T>& s, int i, int j)
-    {
-        if (KIND == KIND_LEAF) return s.Q[i + j * (NX + MT)];
-        if (i < NX && j < NX) return qx(s, i, j);
-        if (i >= NX && j >= NX) return qw(s, i - NX, j - NX);
-        return (T)0;   // Q_xw = 0 at the arrival and master stages
-    }
-    static MHE_DEV T lx(const StageRef<T>& s, int i) { return s.l ? s.l[i] : (T)0; }
-    static MHE_DEV T lw(const StageRef<T>& s, int j)
-    {
-        return (KIND != KIND_UPPER && s.l) ? s.l[NX + j] : (T)0;
-    }
-    static MHE_DEV T a(const StageRef<T>& s, int i) { return s.a ? s.a[i] : (T)0; }
-};
 
 // A -> s.A, B -> s.B, a -> s.e.  FP32 blocks stored in memory (leaf and master
 // stages) move in 16-byte pieces when n is a multiple of four: a column of A or
@@ -242,17 +159,9 @@ MHE_DEV void store_block(T* dst, const T* src, T sgn, int ntail, TF&& tail)
 // finite).  Lane i owns row i of the lower
 // triangle: at column j lane j takes the square root, the lanes below scale
 // their entry of column j and update their own row, so no two lanes write the
-// same entry and a column costs two barriers.  INV (FP32 only) stores 1 / L_jj
-// on the diagonal, the form the FP32 triangular solves use (a multiply per
-// pivot; the refinement absorbs the extra rounding).  FP64 keeps L_jj and
-// divides, which keeps the unrefined FP64 tree within 1e-10 of the oracle.
-template <typename T>
-MHE_DEV T pivot_div(T acc, T gjj)
-{
-    if constexpr (sizeof(T) == 4) return acc * gjj;   // gjj = 1 / L_jj
-    else return acc / gjj;
-}
-
+// same entry and a column costs two barriers.  INV stores 1 / L_jj on the
+// diagonal, the form the triangular solves use: a multiply per pivot, where an FP64
+// division costs as much as six FP64 products of a warp (407 against 64 cycles).
 template <typename T, int NX, int M, bool INV = false>
 MHE_DEV bool chol_inplace(Ws<T, NX>& s, T* Gm, double piv_rel)
 {
@@ -260,7 +169,7 @@ MHE_DEV bool chol_inplace(Ws<T, NX>& s, T* Gm, double piv_rel)
     constexpr int ld = Ws<T, NX>::ld;
     if constexpr (M <= 32) {
         // rows in the registers of one warp, columns passed by shuffles
-        team_chol<T, M, INV && sizeof(T) == 4>(Gm, ld, piv_rel, s.sc + 1);
+        team_chol<T, M, INV>(Gm, ld, piv_rel, s.sc + 1);
         return s.sc[1] != 0;
     }
     wone([&](int) { s.sc[1] = 0; });
@@ -273,7 +182,7 @@ MHE_DEV bool chol_inplace(Ws<T, NX>& s, T* Gm, double piv_rel)
             if (!(d > (T)(piv_rel * (double)mabs(g0)))) { s.sc[1] = 1; d = 1; }
             const T l = msqrt(d);
             s.sc[2] = l;
-            Gm[j + j * ld] = (INV && sizeof(T) == 4) ? (T)1 / l : l;
+            Gm[j + j * ld] = INV ? (T)1 / l : l;
         });
         const T ljj = s.sc[2];
         wlanes([&](int i) {
@@ -364,7 +273,7 @@ MHE_DEV bool chol_G(Ws<T, NX>& s, double piv_rel)
     return chol_inplace<T, NX, MT, true>(s, s.G, piv_rel);
 }
 
-// ---- blocked triangular solves with the Cholesky factor in s.G ---------------
+// ---- blocked triangular solves with the Cholesky factor in s.G (1 / L_jj on its diagonal) ----
 // Diagonal blocks of SB rows (the largest divisor of M up to 8): a column's
 // solve within a block is a short chain in registers; the coupling between
 // blocks is a team product (wgemm), so every lane works and no register array
@@ -405,7 +314,7 @@ MHE_DEV void lower_solve(const Ws<T, NX>& s, FR&& rhs, FG&& get, FP&& put)
                 T acc = (J > 0) ? get(R0 + i, c) : rhs(R0 + i, c);
 #pragma unroll
                 for (int p = 0; p < i; ++p) acc -= s.G[R0 + i + (R0 + p) * ld] * y[p];
-                y[i] = pivot_div(acc, s.G[R0 + i + (R0 + i) * ld]);
+                y[i] = acc * s.G[R0 + i + (R0 + i) * ld];
             }
 #pragma unroll
             for (int i = 0; i < SB; ++i) put(R0 + i, c, y[i]);
@@ -432,7 +341,7 @@ MHE_DEV void upper_solve(const Ws<T, NX>& s, FR&& rhs, FG&& get, FP&& put)
                 T acc = (J < NB - 1) ? get(R0 + i, c) : rhs(R0 + i, c);
 #pragma unroll
                 for (int p = i + 1; p < SB; ++p) acc -= s.G[R0 + p + (R0 + i) * ld] * y[p];
-                y[i] = pivot_div(acc, s.G[R0 + i + (R0 + i) * ld]);
+                y[i] = acc * s.G[R0 + i + (R0 + i) * ld];
             }
 #pragma unroll
             for (int i = 0; i < SB; ++i) put(R0 + i, c, y[i]);
@@ -458,7 +367,7 @@ MHE_DEV void col_solves(const Ws<T, NX>& s, bool upper, FR&& rhs, FY&& putY, FX&
             T acc = rhs(i, c);
 #pragma unroll
             for (int p = 0; p < i; ++p) acc -= s.G[i + p * ld] * y[p];
-            y[i] = pivot_div(acc, s.G[i + i * ld]);
+            y[i] = acc * s.G[i + i * ld];
             putY(i, c, y[i]);
         }
         if (upper) {
@@ -467,11 +376,40 @@ MHE_DEV void col_solves(const Ws<T, NX>& s, bool upper, FR&& rhs, FY&& putY, FX&
                 T acc = y[i];
 #pragma unroll
                 for (int p = i + 1; p < M; ++p) acc -= s.G[p + i * ld] * y[p];
-                y[i] = pivot_div(acc, s.G[i + i * ld]);
+                y[i] = acc * s.G[i + i * ld];
                 putX(i, c, y[i]);
             }
         }
     });
+}
+
+// L^{-1} of the factor in s.G to dst, transposed (entry (q, j) of the M x M column-major block is
+// L^{-1}(j, q), zero for q > j): the vector passes apply it as two products
+template <typename T, int NX, int M>
+MHE_DEV void store_inverse(Ws<T, NX>& s, T* dst)
+{
+    constexpr int ld = Ws<T, NX>::ld;
+    if constexpr (M <= 24) {
+        wfor(M, [&](int c) {   // column c of L^{-1} in registers
+            T y[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) {
+                T acc = i == c ? (T)1 : (T)0;
+#pragma unroll
+                for (int p = 0; p < i; ++p) acc -= s.G[i + p * ld] * y[p];
+                y[i] = acc * s.G[i + i * ld];
+                dst[c + i * M] = y[i];
+            }
+        });
+    } else {
+        lower_solve<T, NX, M, M>(s, [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); },
+                                 [&](int i, int c) -> T { return s.H[i + c * ld]; },
+                                 [&](int i, int c, T v) { s.H[i + c * ld] = v; });
+        wfor(M * M, [&](int r) {
+            const int c = r % M, i = r / M;
+            dst[r] = i >= c ? s.H[i + c * ld] : (T)0;
+        });
+    }
 }
 
 // ---- the stage products on the tensor cores (tcgen05, kind::tf32) -------------
@@ -907,7 +845,7 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
                                           [&](int i, int j, T v) { s.P[i + j * ld] = v; s.P[j + i * ld] = v; });
     wgemm_tn<T, NX, 1, MT, ld, 0>([&](int i, int) { return s.tv[i] - X::lx(st, i); }, s.K, s.g, (T)1,
                                   [&](int i, int, T v) { s.Psi[i] = v; });
-    if (Lgout) store_block<T, MT, MT, ld, true>(Lgout, s.G, (T)1, 0, [](int) {});
+    if (Lgout) store_inverse<T, NX, MT>(s, Lgout);
     if (!want_v) return bad;
     // e = a + B k
     wgemm<T, NX, 1, MT>([&](int i, int) { return s.e[i]; }, [&](int i, int j) { return s.B[i + j * ld]; },
@@ -943,137 +881,6 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
     s.V = s.Tt;
     s.Tt = tmp;
     return bad;
-}
-
-// ---- bounds-checked build -----------------------------------------------------
-// Compiled with MHE_BOUNDS_CHECK (libmhe_bounds.so), the tree passes check each
-// chunk descriptor against the extents of the level's arrays before the chunk is
-// processed, and each caller-stage index before it is used: an index outside its
-// array records MHE_E_BOUNDS for the instance with (level, chunk, index), and the
-// chunk is skipped or the index replaced by 0, so that no access leaves its
-// array.  Extents < 0 are not checked (serving rings).  The regular build
-// compiles none of it.
-constexpr int kBoundsCode = -10;   // MHE_E_BOUNDS
-
-MHE_DEV bool in_ext(long long i, long long ext) { return ext < 0 || (i >= 0 && i < ext); }
-
-template <typename T>
-MHE_DEV long long bounds_index(const LevelArgs<T>& a, int b, long long i, long long ext)
-{
-#ifdef MHE_BOUNDS_CHECK
-    if (!in_ext(i, ext)) {
-        if (b >= 0 && b < a.ext_batch) record_error(a.status, a.where, b, kBoundsCode, a.level, -1, (int)i);
-        return 0;
-    }
-#else
-    (void)a; (void)b; (void)ext;
-#endif
-    return i;
-}
-
-// the descriptor of chunk ci within the level's extents (always true in the regular build)
-template <typename T>
-MHE_DEV bool chunk_in_bounds(const LevelArgs<T>& a, int ci)
-{
-#ifdef MHE_BOUNDS_CHECK
-    const ChunkDesc cd = a.chunks[ci];
-    if (cd.inst < 0 || cd.inst >= a.ext_batch) return false;   // no instance to report to
-    const LevelInst li = a.li[cd.inst];
-    bool out = true;
-    long long bad = 0;   // the offending index, reported in the stage field of where
-    if (cd.t0 < 0 || cd.len < 1 || cd.t0 + cd.len > li.N) bad = cd.t0;
-    else if (!in_ext(cd.g0, a.ext_S) || !in_ext(cd.g0 + cd.len - 1, a.ext_S)) bad = cd.g0;
-    else if (!in_ext(li.gx, a.ext_X) || !in_ext(li.gx + li.N, a.ext_X)) bad = li.gx;
-    else if (cd.parent >= 0 && (!in_ext(cd.parent, a.ext_S_up) || !in_ext(cd.pw, a.ext_S_up))) bad = cd.parent;
-    else if (cd.parent2 >= 0 && !in_ext(cd.parent2, a.ext_S_up)) bad = cd.parent2;
-    else if (cd.px >= 0 && !in_ext(cd.px, a.ext_X_up)) bad = cd.px;
-    else out = false;
-    if (out) {
-        if (lane_id() == 0) record_error(a.status, a.where, cd.inst, kBoundsCode, a.level, ci, (int)bad);
-        return false;
-    }
-#else
-    (void)a; (void)ci;
-#endif
-    return true;
-}
-
-// ---- stage addressing -------------------------------------------------------
-
-template <typename T, int NX, int NW>
-struct Addr {
-    // level-0 stage t >= 1 of instance b
-    static MHE_DEV StageRef<T> leaf(const LevelArgs<T>& a, int b, int t)
-    {
-        const long long s = bounds_index(a, b, a.in_off[b] + t - 1, a.ext_S_in);
-        const long long sr = bounds_index(a, b, a.rhs_off[b] + t - 1, a.ext_S_in);
-        StageRef<T> r;
-        r.A = a.A + s * NX * NX;
-        r.B = a.B + s * NX * NW;
-        r.Q = a.Q + s * (NX + NW) * (NX + NW);
-        r.Qx = nullptr;
-        r.Qw0 = nullptr;
-        r.l = a.l ? a.l + sr * (NX + NW) : nullptr;
-        r.a = a.a ? a.a + sr * NX : nullptr;
-        return r;
-    }
-    static MHE_DEV StageRef<T> arrival(const LevelArgs<T>& a, int b)
-    {
-        StageRef<T> r;
-        r.A = r.B = r.Q = r.Qx = nullptr;
-        r.Qw0 = a.P0inv + (long long)b * NX * NX;
-        r.l = a.l0 ? a.l0 + (long long)b * 2 * NX : nullptr;
-        r.a = a.a0 ? a.a0 + (long long)b * NX : nullptr;
-        return r;
-    }
-    static MHE_DEV StageRef<T> upper(const LevelArgs<T>& a, long long g)
-    {
-        StageRef<T> r;
-        r.A = a.Ah + g * NX * NX;
-        r.B = a.Bh + g * NX * NX;
-        r.Q = nullptr;
-        r.Qx = a.Qxh + g * NX * NX;
-        r.Qw0 = nullptr;
-        r.l = a.lxh ? a.lxh + g * NX : nullptr;
-        r.a = a.ah ? a.ah + g * NX : nullptr;
-        return r;
-    }
-};
-
-// L2 prefetch of the blocks of level-0 stage t of instance b (t >= 1) a pass
-// reads: PF_A, PF_B, PF_Q, PF_L (l) and PF_AV (a) select them
-enum { PF_A = 1, PF_B = 2, PF_Q = 4, PF_L = 8, PF_AV = 16, PF_ALL = 31 };
-template <typename T, int NX, int NW>
-MHE_DEV void prefetch_leaf(const LevelArgs<T>& a, int b, int t, int what = PF_ALL)
-{
-    if (t < 1) return;
-#ifdef MHE_BOUNDS_CHECK
-    if (!in_ext(a.in_off[b] + t - 1, a.ext_S_in) || !in_ext(a.rhs_off[b] + t - 1, a.ext_S_in)) return;
-#endif
-    const long long s = a.in_off[b] + t - 1;
-    if (what & PF_A) prefetch_l2(a.A + s * NX * NX, (int)(sizeof(T) * NX * NX));
-    if (what & PF_B) prefetch_l2(a.B + s * NX * NW, (int)(sizeof(T) * NX * NW));
-    if (what & PF_Q) prefetch_l2(a.Q + s * (NX + NW) * (NX + NW), (int)(sizeof(T) * (NX + NW) * (NX + NW)));
-    if ((what & PF_L) && a.l) prefetch_l2(a.l + (a.rhs_off[b] + t - 1) * (NX + NW), (int)(sizeof(T) * (NX + NW)));
-    if ((what & PF_AV) && a.a) prefetch_l2(a.a + (a.rhs_off[b] + t - 1) * NX, (int)(sizeof(T) * NX));
-}
-
-// the stored factors P, chol(G), K of level-0 stage g (right-hand-side pass), into L2
-template <typename T, int NX, int NW>
-MHE_DEV void prefetch_rhs_factors(const LevelArgs<T>& a, long long g)
-{
-    prefetch_l2(a.Pst + g * NX * NX, (int)(sizeof(T) * NX * NX));
-    prefetch_l2(a.Lgst + g * NW * NW, (int)(sizeof(T) * NW * NW));
-    prefetch_l2(a.Kst + g * NW * NX, (int)(sizeof(T) * NW * NX));
-}
-
-// the stored factors K, k, L of level-0 stage g (down pass), into L2
-template <typename T, int NX, int NW>
-MHE_DEV void prefetch_factors(const LevelArgs<T>& a, long long g)
-{
-    prefetch_l2(a.Kst + g * NW * NX, (int)(sizeof(T) * NW * NX));
-    prefetch_l2(a.Lst + g * NW * NX, (int)(sizeof(T) * NW * NX));
-    prefetch_l2(a.kst + g * NW, (int)(sizeof(T) * NW));
 }
 
 // ---- Algorithm 4 over one chunk ----------------------------------------------
@@ -1177,368 +984,6 @@ MHE_DEV void reduce_chunk(const LevelArgs<T>& a, int ci, T* smem, TcState* tcs =
         if (!tcs->ok) wone([&](int) { record_error(a.status, a.where, b, -7, a.level, ci, cd.t0); });
     }
     if (bad_t >= 0) wone([&](int) { record_error(a.status, a.where, b, -3, a.level, ci, bad_t); });
-}
-
-// ---- the vector part of Algorithm 4 with stored factors -----------------------
-//
-// The dot products of this pass and of the down pass read their matrix from
-// global memory (L2 after the prefetch); their loops are unrolled in full so a
-// lane has all its loads in flight at once instead of a round trip per eight.
-
-template <typename T, int NX, int MT, int KIND>
-MHE_DEV void rhs_step(Ws<T, NX>& s, const StageRef<T>& st, const T* Pin, const T* Lgin,
-                      const T* Kin, T* kout)
-{
-    constexpr int ld = Ws<T, NX>::ld;
-    using X = Acc<T, KIND, NX, MT>;
-    load_AB<T, NX, MT, KIND>(s, st);
-    wcopy<MT * MT>([&](int idx) { return Lgin[idx]; }, [&](int idx, T v) { s.G[idx % MT + (idx / MT) * ld] = v; });
-    wcopy<MT * NX>([&](int idx) { return Kin[idx]; }, [&](int idx, T v) { s.K[idx % MT + (idx / MT) * ld] = v; });
-    wfor(NX, [&](int i) {
-        T acc = s.Psi[i];
-#pragma unroll
-        for (int p = 0; p < NX; ++p) acc -= Pin[i + p * NX] * s.e[p];
-        s.u[i] = acc;
-    });
-    wfor(MT + NX, [&](int idx) {
-        if (idx < MT) {
-            T acc = -X::lw(st, idx);
-#pragma unroll 8
-            for (int p = 0; p < NX; ++p) acc += s.B[p + idx * ld] * s.u[p];
-            s.g[idx] = acc;
-        } else {
-            int i = idx - MT;
-            T acc = 0;
-#pragma unroll 8
-            for (int p = 0; p < NX; ++p) acc += s.A[p + i * ld] * s.u[p];
-            s.tv[i] = acc;
-        }
-    });
-    // k = G^{-1} g with the stored factor: Lg y = g (y in tmp), Lg^T k = y
-    {
-        auto rhsg = [&](int i, int) -> T { return s.g[i]; };
-        auto gety = [&](int i, int) -> T { return s.tmp[i]; };
-        auto puty = [&](int i, int, T v) { s.tmp[i] = v; };
-        lower_solve<T, NX, MT, 1>(s, rhsg, gety, puty);
-        auto getk = [&](int i, int) -> T { return s.k[i]; };
-        auto putk = [&](int i, int, T v) { s.k[i] = v; };
-        upper_solve<T, NX, MT, 1>(s, gety, getk, putk);
-        wfor(MT, [&](int j) { kout[j] = s.k[j]; });
-    }
-    wfor(NX, [&](int i) {
-        T acc = s.tv[i] - X::lx(st, i);
-#pragma unroll 8
-        for (int q = 0; q < MT; ++q) acc += s.K[q + i * ld] * s.g[q];
-        s.Psi[i] = acc;
-    });
-}
-
-// closed-loop step x <- A x + B (K x + k) + a, x in s.e (in), result in s.u
-template <typename T, int NX, int MT, int KIND>
-MHE_DEV void closed_loop_step(Ws<T, NX>& s, const StageRef<T>& st, const T* Kin, const T* kin)
-{
-    using X = Acc<T, KIND, NX, MT>;
-    wfor(MT, [&](int j) {
-        T acc = kin[j];
-#pragma unroll
-        for (int i = 0; i < NX; ++i) acc += Kin[j + i * MT] * s.e[i];
-        s.tmp[j] = acc;
-    });
-    wfor(NX, [&](int i) {
-        T acc = X::a(st, i);
-#pragma unroll
-        for (int j = 0; j < NX; ++j) acc += X::A(st, i, j) * s.e[j];
-#pragma unroll
-        for (int j = 0; j < MT; ++j) acc += X::B(st, i, j) * s.tmp[j];
-        s.u[i] = acc;
-    });
-    wfor(NX, [&](int i) { s.e[i] = s.u[i]; });
-}
-
-template <typename T, int NX, int NW, bool UPPER>
-MHE_DEV void rhs_chunk(const LevelArgs<T>& a, int ci, T* smem)
-{
-    const ChunkDesc cd = a.chunks[ci];
-    const int b = cd.inst;
-    if (a.active && !a.active[b]) return;
-    const bool last = (cd.flags & CH_LAST) != 0;
-    const bool top = (cd.flags & CH_TOP) != 0;
-    Ws<T, NX> s;
-    s.carve_rhs(smem);
-    const T* lN = UPPER ? (a.lNk ? a.lNk + (long long)b * NX : nullptr)
-                        : (a.lN ? a.lN + (long long)b * NX : nullptr);
-    wfor(NX, [&](int i) { s.Psi[i] = (last && lN) ? -lN[i] : (T)0; });
-    if (!UPPER && cd.t0 + cd.len - 1 >= 1) {
-        prefetch_leaf<T, NX, NW>(a, b, cd.t0 + cd.len - 1, PF_A | PF_B | PF_L | PF_AV);
-        prefetch_rhs_factors<T, NX, NW>(a, cd.g0 + cd.len - 1);
-    }
-    for (int tt = cd.len - 1; tt >= 0; --tt) {
-        const int t = cd.t0 + tt;
-        const long long g = cd.g0 + tt;
-        if (!UPPER && t - 1 >= 1 && tt > 0) {
-            // the next stage of the sweep: its blocks and stored factors
-            prefetch_leaf<T, NX, NW>(a, b, t - 1, PF_A | PF_B | PF_L | PF_AV);
-            prefetch_rhs_factors<T, NX, NW>(a, g - 1);
-        }
-        if (UPPER) {
-            rhs_step<T, NX, NX, KIND_UPPER>(s, Addr<T, NX, NW>::upper(a, g), a.Pst + g * NX * NX,
-                                            a.Lgst + g * NX * NX, a.Kst + g * NX * NX, a.kst + g * NX);
-        } else if (t == 0) {
-            rhs_step<T, NX, NX, KIND_ARRIVAL>(s, Addr<T, NX, NW>::arrival(a, b), a.Pst0 + (long long)b * NX * NX,
-                                              a.Lgst0 + (long long)b * NX * NX, a.Kst0 + (long long)b * NX * NX,
-                                              a.kst0 + (long long)b * NX);
-        } else {
-            rhs_step<T, NX, NW, KIND_LEAF>(s, Addr<T, NX, NW>::leaf(a, b, t), a.Pst + g * NX * NX,
-                                           a.Lgst + g * NW * NW, a.Kst + g * NW * NX, a.kst + g * NW);
-        }
-    }
-    if (!last) {
-        // a^: closed loop from x = 0 over the chunk
-        wfor(NX, [&](int i) { s.e[i] = 0; });
-        for (int tt = 0; tt < cd.len; ++tt) {
-            const int t = cd.t0 + tt;
-            const long long g = cd.g0 + tt;
-            if (UPPER)
-                closed_loop_step<T, NX, NX, KIND_UPPER>(s, Addr<T, NX, NW>::upper(a, g), a.Kst + g * NX * NX,
-                                                        a.kst + g * NX);
-            else if (t == 0)
-                closed_loop_step<T, NX, NX, KIND_ARRIVAL>(s, Addr<T, NX, NW>::arrival(a, b),
-                                                          a.Kst0 + (long long)b * NX * NX, a.kst0 + (long long)b * NX);
-            else
-                closed_loop_step<T, NX, NW, KIND_LEAF>(s, Addr<T, NX, NW>::leaf(a, b, t), a.Kst + g * NW * NX,
-                                                       a.kst + g * NW);
-        }
-        const int copies = cd.parent2 >= 0 ? 2 : 1;
-        wfor(copies * NX, [&](int u) {
-            const long long gp = u < NX ? cd.parent : cd.parent2;
-            const int i = u % NX;
-            a.ah_up[gp * NX + i] = s.e[i];
-            a.lxh_up[gp * NX + i] = -s.Psi[i];
-        });
-    } else if (!top) {
-        wfor(NX, [&](int i) { a.lN_up[(long long)b * NX + i] = -s.Psi[i]; });
-    }
-}
-
-// ---- down pass ---------------------------------------------------------------
-
-template <typename T, int NX, int MT, int KIND>
-MHE_DEV void down_fwd_step(Ws<T, NX>& s, const StageRef<T>& st, const T* Kin, const T* kin,
-                           const T* Lin, bool use_wh, T* xo, T* wo)
-{
-    using X = Acc<T, KIND, NX, MT>;
-    // x_t in s.e, w^ in s.v
-    wfor(MT + NX, [&](int idx) {
-        if (idx < MT) {
-            const int j = idx;
-            T acc = kin[j];
-#pragma unroll
-            for (int i = 0; i < NX; ++i) acc += Kin[j + i * MT] * s.e[i];
-            if (use_wh) {
-#pragma unroll
-                for (int i = 0; i < NX; ++i) acc -= Lin[j + i * MT] * s.v[i];
-            }
-            s.tmp[j] = acc;
-            wo[j] = acc;
-        } else {
-            xo[idx - MT] = s.e[idx - MT];
-        }
-    });
-    wfor(NX, [&](int i) {
-        T acc = X::a(st, i);
-#pragma unroll
-        for (int j = 0; j < NX; ++j) acc += X::A(st, i, j) * s.e[j];
-#pragma unroll
-        for (int j = 0; j < MT; ++j) acc += X::B(st, i, j) * s.tmp[j];
-        s.u[i] = acc;
-    });
-    wfor(NX, [&](int i) { s.e[i] = s.u[i]; });
-}
-
-// sum_j p[j] v[j] over a contiguous column of N entries (v in shared memory): in
-// 16-byte vector loads when p is aligned to them (the whole team takes the same
-// branch: its columns are N entries apart), else entry by entry.  The transposed
-// products (A^T lambda) read a column per lane this way instead of one strided
-// entry per lane and step.
-template <int N, typename T>
-MHE_DEV T col_dot(const T* p, const T* v)
-{
-    constexpr int VW = sizeof(T) == 4 ? (N % 4 == 0 ? 4 : (N % 2 == 0 ? 2 : 1)) : (N % 2 == 0 ? 2 : 1);
-    T acc = (T)0;
-    if (VW > 1 && (reinterpret_cast<uintptr_t>(p) % (VW * sizeof(T))) == 0) {
-#pragma unroll
-        for (int j = 0; j < N; j += VW) {
-            if constexpr (sizeof(T) == 4 && VW == 4) {
-                const float4 q = *reinterpret_cast<const float4*>(p + j);
-                acc += q.x * v[j] + q.y * v[j + 1] + q.z * v[j + 2] + q.w * v[j + 3];
-            } else if constexpr (sizeof(T) == 4 && VW == 2) {
-                const float2 q = *reinterpret_cast<const float2*>(p + j);
-                acc += q.x * v[j] + q.y * v[j + 1];
-            } else if constexpr (sizeof(T) == 8 && VW == 2) {
-                const double2 q = *reinterpret_cast<const double2*>(p + j);
-                acc += q.x * v[j] + q.y * v[j + 1];
-            }
-        }
-        return acc;
-    }
-#pragma unroll
-    for (int j = 0; j < N; ++j) acc += p[j] * v[j];
-    return acc;
-}
-
-// |v| as a float (the size of a correction; float is ample for a norm)
-MHE_DEV float absf_of(float v) { return fabsf(v); }
-MHE_DEV float absf_of(double v) { return abs_to_float(v); }
-
-// lambda_t = Q_x x_t + Q_xw w_t + l_x + A^T lambda_{t+1}  (lambda_{t+1} in s.Psi -> result in s.Psi);
-// with FP64 targets z given, z += (x_t, w_t, lambda_t) and dzm keeps the lane's largest |added value|
-template <typename T, int NX, int MT, int KIND>
-MHE_DEV void down_bwd_step(Ws<T, NX>& s, const StageRef<T>& st, const T* xt, const T* wt, T* lo,
-                           double* zx, double* zw, double* zl, float& dzm)
-{
-    using X = Acc<T, KIND, NX, MT>;
-    wfor(NX, [&](int i) {
-        T acc = X::lx(st, i);
-#pragma unroll
-        for (int j = 0; j < NX; ++j) acc += X::qx(st, i, j) * xt[j];
-#pragma unroll
-        for (int j = 0; j < MT; ++j) acc += X::qxw(st, i, j) * wt[j];
-        // (A^T lambda_{t+1})_i: column i of A (the arrival stage has A = I)
-        if constexpr (KIND == KIND_ARRIVAL) acc += s.Psi[i];
-        else acc += col_dot<NX>(st.A + i * NX, s.Psi);
-        s.u[i] = acc;
-    });
-    wfor(NX + (zx ? NX + MT : 0), [&](int idx) {
-        if (idx < NX) {
-            s.Psi[idx] = s.u[idx];
-            lo[idx] = s.u[idx];
-            if (zl) {
-                zl[idx] += f64_of(s.u[idx]);
-                dzm = fmaxf(dzm, absf_of(s.u[idx]));
-            }
-        } else if (idx < 2 * NX) {
-            zx[idx - NX] += f64_of(xt[idx - NX]);
-            dzm = fmaxf(dzm, absf_of(xt[idx - NX]));
-        } else {
-            zw[idx - 2 * NX] += f64_of(wt[idx - 2 * NX]);
-            dzm = fmaxf(dzm, absf_of(wt[idx - 2 * NX]));
-        }
-    });
-}
-
-template <typename T, int NX, int NW, bool UPPER>
-MHE_DEV void down_chunk(const LevelArgs<T>& a, int ci, T* smem)
-{
-    const ChunkDesc cd = a.chunks[ci];
-    const int b = cd.inst;
-    if (a.active && !a.active[b]) return;
-    const bool last = (cd.flags & CH_LAST) != 0;
-    const bool top = (cd.flags & CH_TOP) != 0;
-    Ws<T, NX> s;
-    s.carve_vectors(smem);
-    const LevelInst li = a.li[b];
-    // x^_i -> s.e, w^_i -> s.v, lambda^_{i+1} -> s.Psi
-    wfor(NX, [&](int i) {
-        s.e[i] = top ? a.x0[(long long)b * NX + i] : a.xd_up[cd.px * NX + i];
-        s.v[i] = last ? (T)0 : a.wd_up[cd.pw * NX + i];
-        s.Psi[i] = last ? (T)0 : a.ld_up[(cd.px + 1) * NX + i];
-    });
-    if (!last && a.piv_up) {
-        // rank-revealing master stage B = Pi L (n x r, zero-padded): the parent solved for
-        // w^'; w^ = Pi [L_11^{-T} w^'_{1..r}; 0], with L(i, j) = B(Pi(i), j)
-        const int* pv = a.piv_up + cd.parent * (NX + 1);
-        const T* Bq = a.Bh_up + cd.parent * NX * NX;
-        wone([&](int) {
-            const int r = pv[NX];
-            for (int i = r - 1; i >= 0; --i) {
-                T acc = s.v[i];
-                for (int p = i + 1; p < r; ++p) acc -= Bq[pv[p] + i * NX] * s.v[p];
-                s.v[i] = acc / Bq[pv[i] + i * NX];
-            }
-            for (int i = 0; i < NX; ++i) s.tmp[i] = s.v[i];
-            for (int i = 0; i < NX; ++i) s.v[pv[i]] = i < r ? s.tmp[i] : (T)0;
-        });
-    } else if (!last) {
-        // the parent solved for w^' = R w^ (square-root master stage): w^ = R^{-1} w^'
-        const T* Lq = a.Bh_up + cd.parent * NX * NX;   // R^T, lower triangular
-        wone([&](int) {
-            for (int i = NX - 1; i >= 0; --i) {
-                T acc = s.v[i];
-                for (int p = i + 1; p < NX; ++p) acc -= Lq[p + i * NX] * s.v[p];
-                s.v[i] = acc / Lq[i + i * NX];
-            }
-        });
-    }
-    auto xo = [&](int t) -> T* { return a.xd + (li.gx + t) * NX; };
-    auto lo = [&](int t) -> T* { return a.ld + (li.gx + t) * NX; };
-    auto wo = [&](int t) -> T* {
-        if (UPPER) return a.wd + (li.gs + t) * NX;
-        return a.wd + a.w_off[b] + (t == 0 ? 0 : NX + (long long)(t - 1) * NW);
-    };
-    auto zxo = [&](int t) -> double* { return a.zx ? a.zx + (li.gx + t) * NX : nullptr; };
-    auto zlo = [&](int t) -> double* { return a.zl ? a.zl + (li.gx + t) * NX : nullptr; };
-    auto zwo = [&](int t) -> double* {
-        return a.zw ? a.zw + a.w_off[b] + (t == 0 ? 0 : NX + (long long)(t - 1) * NW) : nullptr;
-    };
-    for (int tt = 0; tt < cd.len; ++tt) {
-        const int t = cd.t0 + tt;
-        const long long g = cd.g0 + tt;
-        if (!UPPER && tt + 1 < cd.len) {   // the next stage's data and factors, into L2
-            prefetch_leaf<T, NX, NW>(a, b, t + 1, PF_A | PF_B | PF_AV);
-            prefetch_factors<T, NX, NW>(a, g + 1);
-        }
-        if (UPPER)
-            down_fwd_step<T, NX, NX, KIND_UPPER>(s, Addr<T, NX, NW>::upper(a, g), a.Kst + g * NX * NX,
-                                                 a.kst + g * NX, a.Lst + g * NX * NX, !last, xo(t), wo(t));
-        else if (t == 0)
-            down_fwd_step<T, NX, NX, KIND_ARRIVAL>(s, Addr<T, NX, NW>::arrival(a, b),
-                                                   a.Kst0 + (long long)b * NX * NX, a.kst0 + (long long)b * NX,
-                                                   a.Lst0 + (long long)b * NX * NX, !last, xo(t), wo(t));
-        else
-            down_fwd_step<T, NX, NW, KIND_LEAF>(s, Addr<T, NX, NW>::leaf(a, b, t), a.Kst + g * NW * NX,
-                                                a.kst + g * NW, a.Lst + g * NW * NX, !last, xo(t), wo(t));
-    }
-    const int t1 = cd.t0 + cd.len;
-    float dzm = 0.f;   // this lane's largest |value| added into z (the size of a correction)
-    if (last) {
-        // lambda_N = Q_{x,N} x_N + l_N (Q_{x,N} = 0 at level 0)
-        const T* QN = UPPER ? a.QNk + (long long)b * NX * NX : nullptr;
-        const T* lN = UPPER ? (a.lNk ? a.lNk + (long long)b * NX : nullptr)
-                            : (a.lN ? a.lN + (long long)b * NX : nullptr);
-        wfor(NX, [&](int i) {
-            T acc = lN ? lN[i] : (T)0;
-            if (QN) {
-#pragma unroll
-                for (int j = 0; j < NX; ++j) acc += QN[i + j * NX] * s.e[j];
-            }
-            s.Psi[i] = acc;
-            xo(t1)[i] = s.e[i];
-            lo(t1)[i] = acc;
-            if (a.zx) {
-                zxo(t1)[i] += f64_of(s.e[i]);
-                zlo(t1)[i] += f64_of(acc);
-                dzm = fmaxf(dzm, fmaxf(absf_of(s.e[i]), absf_of(acc)));
-            }
-        });
-    }
-    for (int tt = cd.len - 1; tt >= 0; --tt) {
-        const int t = cd.t0 + tt;
-        const long long g = cd.g0 + tt;
-        if (!UPPER && tt > 0) prefetch_leaf<T, NX, NW>(a, b, t - 1, PF_A | PF_Q | PF_L);
-        if (UPPER)
-            down_bwd_step<T, NX, NX, KIND_UPPER>(s, Addr<T, NX, NW>::upper(a, g), xo(t), wo(t), lo(t),
-                                                 zxo(t), zwo(t), zlo(t), dzm);
-        else if (t == 0)
-            down_bwd_step<T, NX, NX, KIND_ARRIVAL>(s, Addr<T, NX, NW>::arrival(a, b), xo(t), wo(t), lo(t),
-                                                   zxo(t), zwo(t), zlo(t), dzm);
-        else
-            down_bwd_step<T, NX, NW, KIND_LEAF>(s, Addr<T, NX, NW>::leaf(a, b, t), xo(t), wo(t), lo(t),
-                                                zxo(t), zwo(t), zlo(t), dzm);
-    }
-    // the instance's largest |correction entry| (non-negative floats order like their bit patterns)
-    if (a.zx && a.dznorm) wlanes([&](int) {
-        if (dzm > 0.f) atomicMax(a.dznorm + b, __float_as_uint(dzm));
-    });
 }
 
 // ---- Algorithm 6 as printed: every subproblem solved again --------------------

@@ -150,7 +150,7 @@ MHE_DEV void st16(float* p, const float (&v)[4])
 }
 MHE_DEV double msqrt(double v) { return sqrt(v); }
 MHE_DEV float mrsqrt(float v) { return rsqrtf(v); }
-MHE_DEV double mrsqrt(double v) { return 1.0 / sqrt(v); }
+MHE_DEV double mrsqrt(double v) { return rsqrt(v); }
 MHE_DEV float msqrt(float v) { return sqrtf(v); }
 MHE_DEV double mabs(double v) { return fabs(v); }
 MHE_DEV float mabs(float v) { return fabsf(v); }
@@ -211,7 +211,7 @@ MHE_DEV void atomic_max_nonneg(double* addr, double v)
 // diagonal scaling of G leaves unchanged) is replaced by 1 and reported:
 // *flag = 1 (else 0), written by lane 0 before the closing team barrier.  INV stores 1 / L_jj on
 // the diagonal and multiplies by it, 1 / L_jj from the reciprocal square root
-// of the pivot (FP32); otherwise L_jj is stored and the column divided (FP64).
+// of the pivot; otherwise L_jj is stored and the column divided.
 template <typename T, int M, bool INV>
 MHE_DEV void team_chol(T* Gm, int ld, double piv_rel, T* flag)
 {
