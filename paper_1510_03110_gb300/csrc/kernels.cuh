@@ -213,57 +213,30 @@ __global__ void __launch_bounds__(256, kResidBlocks) k_resid(ResidArgs<TR> r)
     resid_stage<NX, NW, TR, NY>(r, g, sm[team]);
 }
 
-// The double-float residual (MHE form, FP32 correction solves): the FP32 pipes do
-// about twice the instructions of the FP64 form, and the pairs need more registers;
-// four CTAs per SM give 64 registers a thread
-constexpr int kResidBlocksDF = 4;
-
-// Small shapes (nx <= 8): one resident grid (kResidBlocksDF CTAs per SM) whose
-// teams walk the stages with the grid's stride and ask L2 for their next stage
-// while they evaluate the current one, so that only a team's first stage waits on
-// HBM latency; the next stages of all resident teams fit in L2 several times over
-// (nx = 6: ~30 MB).  Larger shapes keep one stage per team and a grid over all
-// stages: at nx = 24 the resident teams' next stages (~73 MB beside the ~73 MB in
-// use) no longer stay in L2 until they are read (measured: the nx = 24 pass 6.74
-// -> 8.61 ms persistent, the nx = 6 pass 1.62 -> 1.28 ms).  Teams synchronise only
-// within themselves, so their trip counts may differ.
-template <int NX>
-constexpr bool resid_df_persistent() { return NX <= 8; }
-
+// The double-float residual (MHE form, FP32 correction solves): one resident grid of CTAs of up to
+// 128 threads (their workspaces fill an SM's shared memory), whose teams walk the stages.
 template <int NX, int NW, int NY>
-__global__ void __launch_bounds__(256, kResidBlocksDF) k_resid_df(ResidArgs<float> r)
+constexpr int resid_df_teams()
 {
-    __shared__ unsigned long long sm[kMaxTeams][ResidSmem<NX, NW, NY>::count];
-    if (r.any_active && *r.any_active == 0) return;
-    const int team = team_id();
-    if constexpr (resid_df_persistent<NX>()) {
-        const long long stride = (long long)gridDim.x * kMaxTeams;
-        for (long long g = (long long)blockIdx.x * kMaxTeams + team; g < r.nstages; g += stride) {
-            if (g + stride < r.nstages) resid_prefetch_df<NX, NW, NY>(r, g + stride);
-            resid_stage<NX, NW, float, NY>(r, g, sm[team]);
-            wsync();
-        }
-    } else {
-        const long long g = (long long)blockIdx.x * kMaxTeams + team;
-        if (g < r.nstages) resid_stage<NX, NW, float, NY>(r, g, sm[team]);
-    }
+    constexpr int fit = 113 * 1024 / DfWs<NX, NW, NY>::bytes, most = MHE_TEAM >= 64 ? 1 : 64 / MHE_TEAM;
+    return fit < 1 ? 1 : (fit < most ? fit : most);
+}
+template <int NX, int NW, int NY>
+constexpr int resid_df_blocks()
+{
+    constexpr int fit = 228 * 1024 / (resid_df_teams<NX, NW, NY>() * DfWs<NX, NW, NY>::bytes + 1024);
+    return fit > 16 ? 16 : (fit < 1 ? 1 : fit);
 }
 
-// CTAs of the double-float residual that are resident at once on this device
-inline long long resid_df_resident_ctas()
+template <int NX, int NW, int NY>
+__global__ void __launch_bounds__(resid_df_teams<NX, NW, NY>() * MHE_TEAM, resid_df_blocks<NX, NW, NY>())
+    k_resid_df(ResidArgs<float> r)
 {
-    static int sms = 0;
-    if (sms <= 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            sms = v;
-        else {
-            cudaGetLastError();
-            sms = 152;
-        }
-    }
-    return (long long)sms * kResidBlocksDF;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (r.any_active && *r.any_active == 0) return;
+    constexpr int W = resid_df_teams<NX, NW, NY>();
+    StageBlocks it(r, (long long)blockIdx.x * W + team_id(), (long long)gridDim.x * W);
+    resid_df_run<NX, NW, NY>(r, it, smem_raw + (size_t)team_id() * DfWs<NX, NW, NY>::bytes);
 }
 
 // NY = 0: Q form; NY > 0: MHE form (C, R)
@@ -271,15 +244,23 @@ template <int NX, int NW, typename TR, int NY = 0>
 void launch_resid(const ResidArgs<TR>& r, void* stream)
 {
     if (r.nstages <= 0) return;
-    const long long grid = (r.nstages + kMaxTeams - 1) / kMaxTeams;
     if constexpr (NY > 0 && sizeof(TR) == 4) {
         if (r.Ahi) {
-            const long long g =
-                resid_df_persistent<NX>() && grid > resid_df_resident_ctas() ? resid_df_resident_ctas() : grid;
-            k_resid_df<NX, NW, NY><<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(r);
+            constexpr int W = resid_df_teams<NX, NW, NY>();
+            constexpr size_t smem = (size_t)W * DfWs<NX, NW, NY>::bytes;
+            static bool attr = false;
+            if (!attr) {
+                cudaFuncSetAttribute(k_resid_df<NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                attr = true;
+            }
+            const long long blocks = (r.nstages + W - 1) / W;
+            const long long room = (long long)device_sms() * resid_df_blocks<NX, NW, NY>();
+            k_resid_df<NX, NW, NY><<<(unsigned)(blocks < room ? blocks : room), W * MHE_TEAM, smem,
+                                     (cudaStream_t)stream>>>(r);
             return;
         }
     }
+    const long long grid = (r.nstages + kMaxTeams - 1) / kMaxTeams;
     k_resid<NX, NW, TR, NY><<<(unsigned)grid, 256, 0, (cudaStream_t)stream>>>(r);
 }
 

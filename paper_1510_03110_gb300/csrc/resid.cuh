@@ -13,6 +13,7 @@
 #pragma once
 #include "common.h"
 #include "f32conv.h"
+#include "vec.cuh"
 #include "warp.cuh"
 #include "wgemm.cuh"
 
@@ -27,6 +28,16 @@ MHE_DEV TR to_tr(double v)
     else return v;
 }
 
+MHE_DEV int stage_instance(const long long* gs0, int batch, long long gstage)
+{
+    int lo = 0, hi = batch;
+    while (hi - lo > 1) {
+        int mid = (lo + hi) >> 1;
+        if (gs0[mid] <= gstage) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 template <int NX, int NW, int NY = 0>
 struct ResidSmem {
     static constexpr int rows = 5 * NX + NW;
@@ -35,9 +46,7 @@ struct ResidSmem {
     // n and nw >= 3 (every task of the first phase then has one length)
     static constexpr int sp = (NX % NW == 0 && NW >= 3) ? NX / NW : 1;
     static constexpr int mhe_form = 4 * NX + 3 * NW + 3 * NY + 5 + sp * (2 * NX + NY + NW);   // resid_mhe
-    static constexpr int mhe_df = mhe_form + 2 * NX + NW;   // resid_mhe_df: + the split x_t, w_t, lambda_{t+1}
-    static constexpr int qm = q_form > mhe_form ? q_form : mhe_form;
-    static constexpr int count = qm > mhe_df ? qm : mhe_df;   // 8-byte entries
+    static constexpr int count = q_form > mhe_form ? q_form : mhe_form;   // 8-byte entries
 };
 
 // One stage t of instance b: rows of stationarity in x_t and w_t, dynamics
@@ -350,231 +359,507 @@ MHE_DEV float2 df_split(double v)
     return make_float2(h, f32_lo(v, h));
 }
 
-// sum_{j < k} (mh + ml)[j sm] * v[j] into (s, c): one predicated loop, as dot_pred
-template <int KMAX>
-MHE_DEV void dot_df(const float* mh, const float* ml, int sm, const float2* v, int k, float& s, float& c)
+// Two double-float accumulators side by side in packed FP32 instructions (fma.rn.f32x2 and the
+// like work on register pairs): the even and the odd terms of a dot product, half the issue slots.
+using F2 = unsigned long long;
+MHE_DEV F2 pack2(float x, float y)
 {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+MHE_DEV float2 unpack2(F2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+MHE_DEV F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+MHE_DEV F2 add2(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+MHE_DEV F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+MHE_DEV F2 sub2(F2 a, F2 b) { return fma2(b, pack2(-1.f, -1.f), a); }   // exact product: one rounding, as a - b
+
+// the sums s and their compensations: rounding errors of the sums (c) and the products' parts (d)
+struct Df2 {
+    F2 s, c, d;
+    MHE_DEV Df2() : s(0ULL), c(0ULL), d(0ULL) {}
+    // += (ah + al)(bh + bl), nb = -bh: df_acc on both halves
+    MHE_DEV void acc(F2 ah, F2 al, F2 bh, F2 bl, F2 nb)
+    {
+        const F2 p = mul2(ah, bh);
+        const F2 q = fma2(ah, nb, p);   // p - ah bh, exactly
+        const F2 t = add2(s, p);
+        const F2 z = sub2(t, s);
+        const F2 x = sub2(s, sub2(t, z)), y = sub2(p, z);   // x + y = s + p - t, exactly
+        s = t;
+        c = add2(add2(c, x), y);
+        d = sub2(fma2(al, bh, fma2(ah, bl, d)), q);
+    }
+    MHE_DEV void result(float& so, float& co) const
+    {
+        const float2 a = unpack2(s), e = unpack2(c), f = unpack2(d);
+        so = a.x;
+        co = e.x + f.x;
+        df_add(so, co, a.y, e.y + f.y);
+    }
+};
+
+// A vector in shared memory split for the products: hi, lo and -hi parts of n entries each, the parts
+// `pitch` apart
+struct DfVec {
+    const float* p;
+    int pitch;
+};
+
+// sum_{j < L} (mh + ml)[j sm] * v[j] as (s, c); the low parts LO floats behind the high ones.  v starts on
+// an even entry when L is even (pairs are loaded at once)
+template <int L, int LO>
+MHE_DEV float2 dot_df(const float* m, int sm, const DfVec& v)
+{
+    Df2 a;
+    float s, c;
 #pragma unroll
-    for (int j = 0; j < KMAX; ++j)
-        if (j < k) df_acc(s, c, mh[j * sm], ml[j * sm], v[j].x, v[j].y);
+    for (int j = 0; j + 1 < L; j += 2) {
+        const F2 ah = pack2(m[j * sm], m[(j + 1) * sm]), al = pack2(m[j * sm + LO], m[(j + 1) * sm + LO]);
+        F2 bh, bl, nb;
+        if constexpr (L % 2 == 0) {
+            bh = *reinterpret_cast<const F2*>(v.p + j);
+            bl = *reinterpret_cast<const F2*>(v.p + v.pitch + j);
+            nb = *reinterpret_cast<const F2*>(v.p + 2 * v.pitch + j);
+        } else {
+            bh = pack2(v.p[j], v.p[j + 1]);
+            bl = pack2(v.p[v.pitch + j], v.p[v.pitch + j + 1]);
+            nb = pack2(v.p[2 * v.pitch + j], v.p[2 * v.pitch + j + 1]);
+        }
+        a.acc(ah, al, bh, bl, nb);
+    }
+    a.result(s, c);
+    if constexpr (L % 2 != 0)
+        df_acc(s, c, m[(L - 1) * sm], m[(L - 1) * sm + LO], v.p[L - 1], v.p[v.pitch + L - 1]);
+    return make_float2(s, c);
 }
 
-// sum_{j < L} (mh + ml)[j] * v[j] into (s, c) over a contiguous row segment, in
-// loads of VW floats (mh, ml aligned to VW floats)
-template <int L, int VW>
-MHE_DEV void dot_df_row(const float* mh, const float* ml, const float2* v, float& s, float& c)
+// the same over a contiguous segment, in loads of VW floats (m aligned to VW floats)
+template <int L, int LO, int VW>
+MHE_DEV float2 dot_df_col(const float* m, const DfVec& v)
 {
-    static_assert(L % VW == 0 && (VW == 1 || VW == 2 || VW == 4), "whole vectors");
+    if constexpr (VW == 1) {
+        return dot_df<L, LO>(m, 1, v);
+    } else {
+        static_assert(L % VW == 0 && LO % VW == 0, "whole vectors");
+        Df2 a;
 #pragma unroll
-    for (int j = 0; j < L; j += VW) {
-        if constexpr (VW == 4) {
-            const float4 h = *reinterpret_cast<const float4*>(mh + j);
-            const float4 l = *reinterpret_cast<const float4*>(ml + j);
-            df_acc(s, c, h.x, l.x, v[j].x, v[j].y);
-            df_acc(s, c, h.y, l.y, v[j + 1].x, v[j + 1].y);
-            df_acc(s, c, h.z, l.z, v[j + 2].x, v[j + 2].y);
-            df_acc(s, c, h.w, l.w, v[j + 3].x, v[j + 3].y);
-        } else if constexpr (VW == 2) {
-            const float2 h = *reinterpret_cast<const float2*>(mh + j);
-            const float2 l = *reinterpret_cast<const float2*>(ml + j);
-            df_acc(s, c, h.x, l.x, v[j].x, v[j].y);
-            df_acc(s, c, h.y, l.y, v[j + 1].x, v[j + 1].y);
-        } else {
-            df_acc(s, c, mh[j], ml[j], v[j].x, v[j].y);
+        for (int j = 0; j < L; j += VW) {
+            float h[VW], l[VW];
+            ldv(m + j, h);
+            ldv(m + LO + j, l);
+#pragma unroll
+            for (int q = 0; q < VW; q += 2)
+                a.acc(pack2(h[q], h[q + 1]), pack2(l[q], l[q + 1]), *reinterpret_cast<const F2*>(v.p + j + q),
+                      *reinterpret_cast<const F2*>(v.p + v.pitch + j + q),
+                      *reinterpret_cast<const F2*>(v.p + 2 * v.pitch + j + q));
         }
+        float s, c;
+        a.result(s, c);
+        return make_float2(s, c);
     }
 }
 
-// the widest load (4, 2 or 1 floats) that divides the row segment length LP, the
-// column length NX and the stage blocks NX x NX and NX x NW (so that every segment
-// of A and B starts aligned, given 16-byte aligned arrays)
-template <int NX, int NW, int LP>
-constexpr int df_row_width()
+// f(idx) for lo <= idx < hi, lanes round-robin in rounds that are not unrolled (bodies of a hundred
+// instructions and more: the instruction cache), no barrier
+template <class F>
+MHE_DEV void rounds(int lo, int hi, F&& f)
 {
-    return (LP % 4 == 0 && NX % 4 == 0 && (NX * NW) % 4 == 0) ? 4 : ((LP % 2 == 0 && NX % 2 == 0) ? 2 : 1);
+#pragma unroll 1
+    for (int i = lo + lane_id(); i < hi; i += MHE_TEAM) f(i);
 }
 
-// Stage t >= 1 in the MHE form with FP32 correction solves: the tasks of
-// resid_mhe, each a double-float dot product.
+// Shared memory of one team of the double-float residual (bytes).  A stage's float
+// pairs come in two halves through a slot each: C and R (the products u = C x, W w,
+// S^T w, then [S; V] u and C^T e) and A and B ([A | B]^T lambda, A x + B w); while one half
+// is worked on the other's copies, of this stage or the team's next, are in flight.
+// The FP64 vectors read to the end of a stage have a pair of slots of their own.
 template <int NX, int NW, int NY>
-MHE_DEV void resid_mhe_df(const ResidArgs<float>& r, int b, int t, int N, unsigned long long* sm)
-{
-    constexpr int NR = NW + NY, NQ = NX + NW;
-    const long long gx = r.gs0[b] + b;
-    const double* xt = r.x + (gx + t) * NX;
-    const double* xn = xt + NX;
-    const double* lt = r.lam + (gx + t) * NX;
-    const double* ln = lt + NX;
-    const double* wt = r.w + r.w_off[b] + NX + (long long)(t - 1) * NW;
-    const long long s = r.in_off[b] + t - 1;
-    const float *Ah = r.Ahi + s * NX * NX, *Al = r.Alo + s * NX * NX;
-    const float *Bh = r.Bhi + s * NX * NW, *Bl = r.Blo + s * NX * NW;
-    const float *Ch = r.Chi + s * NY * NX, *Cl = r.Clo + s * NY * NX;
-    const float *Rh = r.Rhi + s * NR * NR, *Rl = r.Rlo + s * NR * NR;
-    const double* l = r.l ? r.l + s * NQ : nullptr;
-    const double* a = r.a ? r.a + s * NX : nullptr;
-    const long long so = r.out_off[b] + t - 1;
-    float* rl = r.rl + so * NQ;
-    float* ra = r.ra + so * NX;
-    const bool lastst = (t == N - 1);
-    float2* dA = reinterpret_cast<float2*>(sm);   // A x
-    float2* dB = dA + NX;                         // B w
-    float2* atl = dB + NX;                        // A^T lam_{t+1}
-    float2* cte = atl + NX;                       // C^T e
-    float2* u = cte + NX;                         // C x
-    float2* sw = u + NY;                          // S^T w
-    float2* e = sw + NY;                          // V u - S^T w
-    float2* btl = e + NY;                         // B^T lam_{t+1}
-    float2* ww = btl + NW;                        // W w
-    float2* su = ww + NW;                         // S u
-    float2* vx = su + NW;                         // x_t, w_t, lam_{t+1} as pairs
-    float2* vw = vx + NX;
-    float2* vl = vw + NW;
-    unsigned long long* mx = reinterpret_cast<unsigned long long*>(vl + NX);
-    constexpr int T1 = NX + NY + NX + NW;
-    constexpr int SP = ResidSmem<NX, NW, NY>::sp;
-    constexpr int LP = NX / SP;
-    constexpr int KM = LP > NW ? LP : NW;
-    float2* part = reinterpret_cast<float2*>(mx + 4);   // SP x T1 partial sums
-    // the stage's matrix pairs and right-hand side into L2 now, so that the loads of the
-    // product phases below wait on L2 rather than on HBM (one warp per stage, its phases
-    // separated by barriers: the kernel is bound by memory latency, not bandwidth)
-    prefetch_l2(Ah, (int)sizeof(float) * NX * NX);
-    prefetch_l2(Al, (int)sizeof(float) * NX * NX);
-    prefetch_l2(Bh, (int)sizeof(float) * NX * NW);
-    prefetch_l2(Bl, (int)sizeof(float) * NX * NW);
-    prefetch_l2(Ch, (int)sizeof(float) * NY * NX);
-    prefetch_l2(Cl, (int)sizeof(float) * NY * NX);
-    prefetch_l2(Rh, (int)sizeof(float) * NR * NR);
-    prefetch_l2(Rl, (int)sizeof(float) * NR * NR);
-    if (l) prefetch_l2(l, (int)sizeof(double) * NQ);
-    if (a) prefetch_l2(a, (int)sizeof(double) * NX);
-    wfor(2 * NX + NW, [&](int k) {
-        if (k < NX) vx[k] = df_split(xt[k]);
-        else if (k < NX + NW) vw[k - NX] = df_split(wt[k - NX]);
-        else vl[k - NX - NW] = df_split(ln[k - NX - NW]);
-        if (k == 0) mx[0] = mx[1] = mx[2] = 0ULL;
-    });
-    // the tasks: the column-strided pieces of A x and C x first, then the contiguous row
-    // pieces of A^T lam and B^T lam (vector loads), then the length-nw products: warps
-    // mostly run tasks of one kind
-    constexpr int TS = (NX + NY) * SP, TC = (NX + NW) * SP;
-    constexpr int VW = df_row_width<NX, NW, LP>();
-    wfor(T1 * SP + NX + NW + NY, [&](int k) {
-        const float *mh, *ml;
-        const float2* v;
-        float2* o;
-        int st, len = LP;
-        if (k < TS) {
-            const int q = k % (NX + NY), c = k / (NX + NY), j0 = c * LP;
-            o = part + c * T1 + q;
-            if (q < NX) { mh = Ah + q + j0 * NX; ml = Al + q + j0 * NX; st = NX; v = vx + j0; }
-            else { mh = Ch + (q - NX) + j0 * NY; ml = Cl + (q - NX) + j0 * NY; st = NY; v = vx + j0; }
-        } else if (k < TS + TC) {
-            const int q = (k - TS) % (NX + NW), c = (k - TS) / (NX + NW), j0 = c * LP;
-            o = part + c * T1 + NX + NY + q;
-            if (q < NX) { mh = Ah + q * NX + j0; ml = Al + q * NX + j0; }
-            else { mh = Bh + (q - NX) * NX + j0; ml = Bl + (q - NX) * NX + j0; }
-            float ds = 0.f, dc = 0.f;
-            dot_df_row<LP, VW>(mh, ml, vl + j0, ds, dc);
-            *o = make_float2(ds, dc);
-            return;
-        } else {
-            const int q = k - T1 * SP;
-            len = NW;
-            if (q < NX) { mh = Bh + q; ml = Bl + q; st = NX; v = vw; o = dB + q; }
-            else if (q < NX + NW) { mh = Rh + (q - NX); ml = Rl + (q - NX); st = NR; v = vw; o = ww + (q - NX); }
-            else {
-                // S^T w: the first nw entries of column nw + i of R, contiguous
-                const int i = q - NX - NW;
-                float ds = 0.f, dc = 0.f;
-                dot_df_row<NW, df_row_width<NR, NR, NW>()>(Rh + (NW + i) * NR, Rl + (NW + i) * NR, vw, ds, dc);
-                sw[i] = make_float2(ds, dc);
-                return;
+struct DfWs {
+    static constexpr int NR = NW + NY, NQ = NX + NW;
+    // the length-n products are cut into SP segments of length LP (= nw when it divides n), so
+    // that the tasks of a phase have about one length
+    static constexpr int SP = NX % NW == 0 ? NX / NW : 1, LP = NX / SP;
+    static constexpr int ldA = pick_ld(NX, vec_of<float>(NX)), ldC = pick_ld(NY, vec_of<float>(NY));
+    static constexpr int vA = LP % vec_of<float>(NX) == 0 ? vec_of<float>(NX) : (LP % 2 == 0 && ldA % 2 == 0 ? 2 : 1);
+    // floats: [A | B] hi, then lo
+    static constexpr int oB = ldA * NX, abl = round_to(ldA * NQ, 4), ab = 2 * abl;
+    // floats: C and R hi, then lo
+    static constexpr int oR = round_to(ldC * NX, 4), crl = oR + round_to(NR * NR, 4), cr = 2 * crl;
+    // doubles: x_t, w_t, lambda_{t+1}, split at once; lambda_t, x_{t+1}, l, a, read at the end (two slots)
+    static constexpr int vec1 = round_to(NQ + NX, 2);
+    static constexpr int oxn = NX, ol = oxn + NX, oa = ol + NQ, vec2 = round_to(oa + NX, 2);
+    // split vectors (floats, three parts each): (x, w) and lambda_{t+1}; u and e (in col's place: they are
+    // done with before col is begun).  w follows x at once when it makes the products' last segment
+    static constexpr int sw0 = LP == NW ? NX : round_to(NX, 2);
+    static constexpr int olam = round_to(sw0 + NW, 4), pz = olam + round_to(NX, 4), py = round_to(NY, 4), split = 3 * pz;
+    // float2: partial sums and products (cx, ww, sw are done with before row is begun)
+    static constexpr int row = 0, cx = 0, ww = row + (SP + 1) * NX, sw = cx + SP * NY, col = ww + NW,
+                         su = col + max_int(SP * NQ, 3 * py),
+                         cte = su + NW, pairs = round_to(cte + NX, 2);
+    static_assert(SP * NY + NY <= (SP + 1) * NX, "cx and sw fit row");
+    static constexpr int bytes = (4 * (ab + cr + split) + 8 * (vec1 + 2 * vec2) + 8 * pairs + 15) / 16 * 16;
+};
+
+// the stages of a team's share, next(b, t, N) one after another (false: no more): blocks of
+// stages dealt round-robin over all teams, instances that no longer refine left out
+struct StageBlocks {
+    const long long* gs0;
+    const int* active;
+    int batch, len, b = 0;
+    long long blk, stride, total, g = 0, end = 0, g0 = 0, g1 = 0;
+    template <typename TR>
+    MHE_DEV StageBlocks(const ResidArgs<TR>& r, long long team, long long teams)
+        : gs0(r.gs0), active(r.active), batch(r.batch), blk(team - teams), stride(teams), total(r.nstages)
+    {
+        // eight stages a block (an instance's offsets are looked up once a block), fewer when that
+        // would leave teams without a block
+        const long long most = (total + teams - 1) / teams;
+        len = most < 8 ? (int)most : 8;
+    }
+    MHE_DEV bool next(int& bo, int& t, int& N)
+    {
+        for (;;) {
+            if (g >= end) {
+                blk += stride;
+                g = blk * len;
+                if (g >= total) return false;
+                end = g + len < total ? g + len : total;
+                b = stage_instance(gs0, batch, g);
+                g0 = gs0[b];
+                g1 = gs0[b + 1];
             }
+            while (g >= g1) {
+                ++b;
+                g0 = g1;
+                g1 = gs0[b + 1];
+            }
+            if (active && !active[b]) {
+                g = g1;
+                continue;
+            }
+            bo = b;
+            t = (int)(g - g0);
+            N = (int)(g1 - g0);
+            ++g;
+            return true;
         }
-        float ds = 0.f, dc = 0.f;
-        dot_df<KM>(mh, ml, st, v, len, ds, dc);
-        *o = make_float2(ds, dc);
-    });
-    // the length-n products from their pieces; C x normalised (it is the next phase's vector)
-    wfor(T1, [&](int q) {
-        float ds = part[q].x, dc = part[q].y;
+    }
+};
+
+// the stages team, team + teams, .. of one instance
+struct StageStride {
+    int b, t, teams, N;
+    MHE_DEV bool next(int& bo, int& to, int& No)
+    {
+        if (t >= N) return false;
+        bo = b;
+        to = t;
+        No = N;
+        t += teams;
+        return true;
+    }
+};
+
+// running maxima of |r| (float bits), |z|, |b| (double bits) of one instance, merged into its norms at once
+struct NormMax {
+    unsigned r = 0;
+    unsigned long long z = 0, b = 0;
+    MHE_DEV void see_r(float v) { const unsigned u = __float_as_uint(v) & 0x7fffffffu; r = u > r ? u : r; }
+    MHE_DEV void see_z(double v) { const unsigned long long u = abs_bits(v); z = u > z ? u : z; }
+    MHE_DEV void see_b(double v) { const unsigned long long u = abs_bits(v); b = u > b ? u : b; }
+    MHE_DEV void flush(unsigned long long* norms)
+    {
+        constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32;
+        const unsigned mask =
+            CW == 32 ? 0xffffffffu : (((1u << CW) - 1u) << ((threadIdx.x & 31) & ~(CW - 1)));
+        unsigned long long m[3] = {abs_bits(f64_of(__uint_as_float(r))), z, b};
 #pragma unroll
-        for (int c = 1; c < SP; ++c) df_add(ds, dc, part[c * T1 + q].x, part[c * T1 + q].y);
-        if (q < NX) dA[q] = make_float2(ds, dc);
-        else if (q < NX + NY) u[q - NX] = df_norm(ds, dc);
-        else if (q < 2 * NX + NY) atl[q - NX - NY] = make_float2(ds, dc);
-        else btl[q - 2 * NX - NY] = make_float2(ds, dc);
-    });
-    // e = V u - S^T w (normalised: the next phase's vector), S u
-    wfor(NY + NW, [&](int k) {
-        const float *mh, *ml;
-        float ds, dc;
-        if (k < NY) { mh = Rh + NW + k + NW * NR; ml = Rl + NW + k + NW * NR; ds = -sw[k].x; dc = -sw[k].y; }
-        else { mh = Rh + (k - NY) + NW * NR; ml = Rl + (k - NY) + NW * NR; ds = 0.f; dc = 0.f; }
-        dot_df<NY>(mh, ml, NR, u, NY, ds, dc);
-        if (k < NY) e[k] = df_norm(ds, dc);
-        else su[k - NY] = make_float2(ds, dc);
-    });
-    wfor(NX, [&](int i) {
-        float ds = 0.f, dc = 0.f;
-        dot_df_row<NY, df_row_width<NY, NX, NY>()>(Ch + i * NY, Cl + i * NY, e, ds, dc);   // column i of C
-        cte[i] = make_float2(ds, dc);
-    });
-    unsigned long long m0 = 0, m1 = 0, m2 = 0;
-    const int nrow = NQ + NX + (lastst ? NX : 0);
-    const double* xN = r.x + (gx + N) * NX;
-    const double* lamN = r.lam + (gx + N) * NX;
-    const float2 zero2 = make_float2(0.f, 0.f);
-    wfor(nrow, [&](int i) {
-        float2 p1, p2;
-        const double *p3, *p4, *z1, *z2;
-        const double zd = 0.0;
-        float* dst;
-        if (i < NX) {
-            p1 = cte[i]; p2 = atl[i]; p3 = lt + i; p4 = l ? l + i : &zd;
-            z1 = xt + i; z2 = lt + i; dst = rl + i;
-        } else if (i < NQ) {
-            const int q = i - NX;
-            p1 = ww[q]; p2 = btl[q]; p4 = l ? l + i : &zd;
-            p3 = &zd;
-            z1 = wt + q; z2 = &zd; dst = rl + i;
-        } else if (i < NQ + NX) {
-            const int ii = i - NQ;
-            p1 = dA[ii]; p2 = dB[ii]; p3 = xn + ii; p4 = a ? a + ii : &zd;
-            z1 = &zd; z2 = &zd; dst = ra + ii;
-        } else {
-            // terminal rows with Q_{x,N} = 0, l_N = 0: r = lambda_N
-            const int ii = i - NQ - NX;
-            p1 = zero2; p2 = zero2; p3 = lamN + ii; p4 = &zd;
-            z1 = xN + ii; z2 = lamN + ii; dst = r.rlN + (long long)b * NX + ii;
+        for (int k = 0; k < 3; ++k) {
+#pragma unroll
+            for (int d = CW / 2; d > 0; d /= 2) {
+                const unsigned long long o = __shfl_xor_sync(mask, m[k], d, CW);
+                m[k] = o > m[k] ? o : m[k];
+            }
+            if ((lane_id() & (CW - 1)) == 0 && m[k]) atomic_max_u64(norms + k, m[k]);
         }
-        // r = -(l + K z): p4 + (p1 + p2 - p3), with the S u term of the w rows subtracted
-        const float2 v3 = df_split(*p3), v4 = df_split(*p4);
-        float ds = v4.x, dc = v4.y;
-        df_add(ds, dc, p1.x, p1.y);
-        df_add(ds, dc, p2.x, p2.y);
-        df_add(ds, dc, -v3.x, -v3.y);
-        if (i >= NX && i < NQ) df_add(ds, dc, -su[i - NX].x, -su[i - NX].y);
-        const float sum = ds + dc;
-        *dst = sum;
-        const unsigned long long rr = abs_bits(f64_of(sum)), bb = abs_bits(*p4);
-        const unsigned long long za = abs_bits(*z1), zb = abs_bits(*z2);
-        const unsigned long long zz = za > zb ? za : zb;
-        m0 = rr > m0 ? rr : m0;
-        m1 = zz > m1 ? zz : m1;
-        m2 = bb > m2 ? bb : m2;
+        r = 0;
+        z = b = 0;
+    }
+};
+
+// The arrival stage t = 0 (A_0 = B_0 = I, Q_0 = diag(0, P~0^{-1}), l_0 = a_0 = 0) in FP64, and the initial rows
+template <int NX>
+MHE_DEV void resid_arrival(const ResidArgs<float>& r, int b, int N, NormMax& mx)
+{
+    const long long gx = r.gs0[b] + b;
+    const double *xt = r.x + gx * NX, *lt = r.lam + gx * NX, *wt = r.w + r.w_off[b];
+    const double* P0 = r.P0inv + (long long)b * NX * NX;
+    each<NX>([&](int i) {
+        const double x = xt[i], xn = xt[NX + i], l = lt[i], ln = lt[NX + i], w = wt[i], x0 = r.x0[(long long)b * NX + i];
+        double q = ln;
+#pragma unroll 4
+        for (int j = 0; j < NX; ++j) q = fma(P0[i + j * NX], wt[j], q);
+        const float rx = f32_rn(ln - l), rw = f32_rn(q), rd = f32_rn(x + w - xn), ri = f32_rn(x0 - x);
+        r.rl0[(long long)b * 2 * NX + i] = rx;
+        r.rl0[(long long)b * 2 * NX + NX + i] = rw;
+        r.ra0[(long long)b * NX + i] = rd;
+        r.rx0[(long long)b * NX + i] = ri;
+        mx.see_r(rx); mx.see_r(rw); mx.see_r(rd); mx.see_r(ri);
+        mx.see_z(x); mx.see_z(l); mx.see_z(w);
+        mx.see_b(x0);
+        if (N == 1) {   // terminal rows: -(0 - lambda_N)
+            r.rlN[(long long)b * NX + i] = f32_rn(-ln);
+            mx.see_r(f32_rn(ln));
+            mx.see_z(xn); mx.see_z(ln);
+        }
     });
-    atomic_max_u64(mx + 0, m0);
-    atomic_max_u64(mx + 1, m1);
-    atomic_max_u64(mx + 2, m2);
-    wsync();
-    wone([&](int) {
-        atomic_max_u64(r.norms + 3LL * b + 0, mx[0]);
-        atomic_max_u64(r.norms + 3LL * b + 1, mx[1]);
-        atomic_max_u64(r.norms + 3LL * b + 2, mx[2]);
-    });
+}
+
+// The MHE-form residual with FP32 correction solves over the stages `it` yields.
+// Per stage t >= 1 (the tasks of resid_mhe, each a double-float dot product):
+//   C and R:  u = C x,  W w,  S^T w;   then  S u,  e = V u - S^T w;   then  C^T e;
+//   A and B:  A x + B w,  A^T lambda_{t+1},  B^T lambda_{t+1};   then the rows.
+// What bounds it: HBM has 15.4 KB a stage to deliver at nx = 24 (1.2 ms for 535k stages); the products are
+// 2880 double-float terms of 12 packed instructions for two, so the nine to ten teams an SM holds
+// are now bound by the latency of their dependent sums (ncu: 46% issue, 51% DRAM).  Full pass, before
+// (a stage's tasks read straight from global memory, scalar instructions) and after: nx = 24, 535k
+// stages, 2.63 -> 2.06 ms; nx = 12, 1.05M stages, 2.13 -> 1.26 ms; nx = 6, 1.10M stages, 0.97 -> 0.54 ms; nx = 64,
+// 131k stages, 4.09 -> 3.96 ms.
+template <int NX, int NW, int NY, class IT>
+MHE_DEV void resid_df_run(const ResidArgs<float>& r, IT& it, unsigned char* smem)
+{
+    using S = DfWs<NX, NW, NY>;
+    constexpr int NR = S::NR, NQ = S::NQ, SP = S::SP, LP = S::LP, ldA = S::ldA, ldC = S::ldC;
+    constexpr int aB = piece_of(4 * S::oB), aR = piece_of(4 * NR * NR);
+    float* cr = reinterpret_cast<float*>(smem);
+    float* ab = cr + S::cr;
+    float* sz = ab + S::ab;           // split (x, w), lambda
+    double* vi = reinterpret_cast<double*>(sz + S::split);
+    double* vec0 = vi + S::vec1;
+    float2* pr = reinterpret_cast<float2*>(vec0 + 2 * S::vec2);
+    float* su = reinterpret_cast<float*>(pr + S::col);   // split u, e
+    auto put = [](float* p, int pitch, int k, const float2& v) {
+        p[k] = v.x;
+        p[pitch + k] = v.y;
+        p[2 * pitch + k] = -v.x;
+    };
+    auto zv = [&](int k) { return DfVec{sz + k, S::pz}; };
+    auto yv = [&](int e) { return DfVec{su + e * 3 * S::py, S::py}; };
+    NormMax mx;
+    int b = 0, t = 0, N = 0;
+    bool have;
+    // the team's next stage t >= 1; arrival stages are evaluated on the way
+    auto advance = [&]() {
+        for (;;) {
+            have = it.next(b, t, N);
+            if (!have || t > 0) return;
+            NormMax am;
+            resid_arrival<NX>(r, b, N, am);
+            am.flush(r.norms + 3LL * b);
+        }
+    };
+    auto load_cr = [&](double* v) {
+        const long long s = r.in_off[b] + t - 1, gx = r.gs0[b] + b + t;
+        async_block<float, NY, NX, ldC>(cr, r.Chi + s * NY * NX);
+        async_block<float, NR, NR, NR, NR, aR>(cr + S::oR, r.Rhi + s * NR * NR);
+        async_block<float, NY, NX, ldC>(cr + S::crl, r.Clo + s * NY * NX);
+        async_block<float, NR, NR, NR, NR, aR>(cr + S::crl + S::oR, r.Rlo + s * NR * NR);
+        async_vec<double, NX>(vi, r.x + gx * NX);
+        async_vec<double, NW>(vi + NX, r.w + r.w_off[b] + NX + (long long)(t - 1) * NW);
+        async_vec<double, NX>(vi + NQ, r.lam + (gx + 1) * NX);
+        async_vec<double, NX>(v, r.lam + gx * NX);
+        async_vec<double, NX>(v + S::oxn, r.x + (gx + 1) * NX);
+        async_vec<double, NQ>(v + S::ol, r.l ? r.l + s * NQ : nullptr);
+        async_vec<double, NX>(v + S::oa, r.a ? r.a + s * NX : nullptr);
+    };
+    auto load_ab = [&]() {
+        const long long s = r.in_off[b] + t - 1;
+        async_block<float, NX, NX, ldA>(ab, r.Ahi + s * NX * NX);
+        async_block<float, NX, NW, ldA, NX, aB>(ab + S::oB, r.Bhi + s * NX * NW);
+        async_block<float, NX, NX, ldA>(ab + S::abl, r.Alo + s * NX * NX);
+        async_block<float, NX, NW, ldA, NX, aB>(ab + S::abl + S::oB, r.Blo + s * NX * NW);
+    };
+    advance();
+    int par = 0;
+    if (have) load_cr(vec0);
+    cp_commit();
+    while (have) {
+        const double* v = vec0 + par * S::vec2;
+        load_ab();
+        cp_commit();
+        const int sb = b, st = t;
+        const bool lastst = t == N - 1;
+        cp_wait<1>();
+        wsync();
+        // ---- C and R
+        rounds(0, NQ + NX, [&](int k) {
+            const double z = vi[k];
+            put(sz, S::pz, k < NX ? k : (k < NQ ? S::sw0 + k - NX : S::olam + k - NQ), df_split(z));
+            if (k < NQ || lastst) mx.see_z(z);
+        });
+        wsync();
+        // segments of C x, then W w and S^T w (the first nw entries of column nw + k of R)
+        if constexpr (LP == NW) {
+            rounds(0, NY * SP + NW + NY, [&](int k) {
+                const float* m;
+                int sm, j0, o;
+                if (k < NY * SP) {
+                    j0 = (k / NY) * LP;
+                    m = cr + k % NY + j0 * ldC;
+                    sm = ldC;
+                    o = S::cx + k;
+                } else if (k < NY * SP + NW) {
+                    const int q = k - NY * SP;
+                    m = cr + S::oR + q;
+                    sm = NR;
+                    j0 = NX;
+                    o = S::ww + q;
+                } else {
+                    const int q = k - NY * SP - NW;
+                    m = cr + S::oR + (NW + q) * NR;
+                    sm = 1;
+                    j0 = NX;
+                    o = S::sw + q;
+                }
+                pr[o] = dot_df<LP, S::crl>(m, sm, zv(j0));
+            });
+        } else {
+            rounds(0, NY * SP, [&](int k) {
+                const int j0 = (k / NY) * LP;
+                pr[S::cx + k] = dot_df<LP, S::crl>(cr + k % NY + j0 * ldC, ldC, zv(j0));
+            });
+            rounds(0, NR, [&](int k) {
+                const bool w = k < NW;
+                pr[w ? S::ww + k : S::sw + k - NW] =
+                    dot_df<NW, S::crl>(cr + S::oR + (w ? k : k * NR), w ? NR : 1, zv(S::sw0));
+            });
+        }
+        wsync();
+        rounds(0, NY, [&](int k) {
+            float s = pr[S::cx + k].x, c = pr[S::cx + k].y;
+#pragma unroll
+            for (int q = 1; q < SP; ++q) df_add(s, c, pr[S::cx + q * NY + k].x, pr[S::cx + q * NY + k].y);
+            put(su, S::py, k, df_norm(s, c));
+        });
+        wsync();
+        rounds(0, NR, [&](int k) {   // row k of [S; V] u;  e = V u - S^T w
+            const float2 d = dot_df<NY, S::crl>(cr + S::oR + k + NW * NR, NR, yv(0));
+            if (k < NW) {
+                pr[S::su + k] = d;
+            } else {
+                float s = d.x, c = d.y;
+                df_add(s, c, -pr[S::sw + k - NW].x, -pr[S::sw + k - NW].y);
+                put(su + 3 * S::py, S::py, k - NW, df_norm(s, c));
+            }
+        });
+        wsync();
+        rounds(0, NX, [&](int i) {   // C^T e
+            pr[S::cte + i] = dot_df_col<NY, S::crl, NY % 2 == 0 ? vec_of<float>(NY) : 1>(cr + i * ldC, yv(1));
+        });
+        wsync();   // the C and R slot is free
+        advance();
+        par ^= 1;
+        if (have) load_cr(vec0 + par * S::vec2);
+        cp_commit();
+        cp_wait<1>();
+        wsync();
+        // ---- A and B: row i of [A | B] with (x, w), in segments (the last one B w)
+        constexpr int nrow = NX * (SP + 1), ncol = NQ * SP, T = MHE_TEAM;
+        // whole rounds of either kind, then the rest of both in one round with the stride chosen per lane
+        constexpr bool mixed = LP == NW && nrow % T + ncol % T <= T && nrow % T > 0 && ncol % T > 0;
+        constexpr int row1 = mixed ? nrow / T * T : nrow, col1 = mixed ? ncol / T * T : ncol;
+        rounds(0, row1, [&](int k) {
+            const int i = k % NX, j0 = (k / NX) * LP;
+            if constexpr (LP == NW) {
+                pr[S::row + k] = dot_df<LP, S::abl>(ab + i + j0 * ldA, ldA, zv(j0));
+            } else {
+                if (k < NX * SP) pr[S::row + k] = dot_df<LP, S::abl>(ab + i + j0 * ldA, ldA, zv(j0));
+                else pr[S::row + k] = dot_df<NW, S::abl>(ab + S::oB + i, ldA, zv(S::sw0));
+            }
+        });
+        // column i of [A | B] with lambda_{t+1}, in segments
+        rounds(0, col1, [&](int k) {
+            const int i = k % NQ, j0 = (k / NQ) * LP;
+            pr[S::col + k] = dot_df_col<LP, S::abl, LP % 2 == 0 ? S::vA : 1>(ab + i * ldA + j0, zv(S::olam + j0));
+        });
+        if constexpr (mixed) {
+            rounds(0, nrow - row1 + ncol - col1, [&](int k) {
+                const bool rw = k < nrow - row1;
+                const int q = rw ? row1 + k : col1 + k - (nrow - row1);
+                const int i = rw ? q % NX : q % NQ, j0 = (rw ? q / NX : q / NQ) * LP;
+                pr[rw ? S::row + q : S::col + q] = dot_df<LP, S::abl>(ab + (rw ? i + j0 * ldA : i * ldA + j0),
+                                                                     rw ? ldA : 1, zv(rw ? j0 : S::olam + j0));
+            });
+        }
+        wsync();
+        // ---- the rows: r = -(l + K z)
+        const long long so = r.out_off[sb] + st - 1;
+        float *rl = r.rl + so * NQ, *ra = r.ra + so * NX;
+        rounds(0, NX, [&](int i) {   // C^T e + A^T lambda_{t+1} - lambda_t + l_x
+            const double l = v[S::ol + i], lt = v[i];
+            const float2 v4 = df_split(l - lt);
+            float s = v4.x, c = v4.y;
+            df_add(s, c, pr[S::cte + i].x, pr[S::cte + i].y);
+#pragma unroll
+            for (int q = 0; q < SP; ++q) df_add(s, c, pr[S::col + q * NQ + i].x, pr[S::col + q * NQ + i].y);
+            rl[i] = s + c;
+            mx.see_r(s + c);
+            mx.see_z(lt);
+            mx.see_b(l);
+        });
+        rounds(0, NW, [&](int i) {   // W w - S u + B^T lambda_{t+1} + l_w
+            const double l = v[S::ol + NX + i];
+            const float2 v4 = df_split(l);
+            float s = v4.x, c = v4.y;
+            df_add(s, c, pr[S::ww + i].x, pr[S::ww + i].y);
+#pragma unroll
+            for (int q = 0; q < SP; ++q) df_add(s, c, pr[S::col + q * NQ + NX + i].x, pr[S::col + q * NQ + NX + i].y);
+            df_add(s, c, -pr[S::su + i].x, -pr[S::su + i].y);
+            rl[NX + i] = s + c;
+            mx.see_r(s + c);
+            mx.see_b(l);
+        });
+        rounds(0, NX, [&](int i) {   // A x + B w - x_{t+1} + a
+            const double a = v[S::oa + i], xn = v[S::oxn + i];
+            const float2 v4 = df_split(a - xn);
+            float s = v4.x, c = v4.y;
+#pragma unroll
+            for (int q = 0; q <= SP; ++q) df_add(s, c, pr[S::row + q * NX + i].x, pr[S::row + q * NX + i].y);
+            ra[i] = s + c;
+            mx.see_r(s + c);
+            mx.see_b(a);
+            if (lastst) {   // terminal rows with Q_{x,N} = 0, l_N = 0: r = lambda_N
+                const float ln = sz[S::olam + i] + sz[S::pz + S::olam + i];
+                r.rlN[(long long)sb * NX + i] = -ln;
+                mx.see_r(ln);
+                mx.see_z(xn);
+            }
+        });
+        if (!have || b != sb) mx.flush(r.norms + 3LL * sb);
+        wsync();   // the A and B slot and the products are free
+    }
+    cp_wait<0>();
 }
 
 // Stage t >= 1 with the assembled Q: the same rows as resid_rows, as dot
@@ -671,45 +956,6 @@ MHE_DEV void resid_q(const ResidArgs<TR>& r, int b, int t, int N, unsigned long 
     });
 }
 
-MHE_DEV int stage_instance(const long long* gs0, int batch, long long gstage)
-{
-    int lo = 0, hi = batch;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (gs0[mid] <= gstage) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-// The stage a team evaluates next, asked into L2 while it evaluates the current
-// one (the double-float MHE form: the stage's matrix pairs, l, a and the iterate's
-// vectors).  Every address lies in the arrays' extents for the stage; the
-// arrival stage is left out.
-template <int NX, int NW, int NY>
-MHE_DEV void resid_prefetch_df(const ResidArgs<float>& r, long long gstage)
-{
-    constexpr int NR = NW + NY, NQ = NX + NW;
-    const int b = stage_instance(r.gs0, r.batch, gstage);
-    if (r.active && !r.active[b]) return;
-    const int t = (int)(gstage - r.gs0[b]);
-    if (t == 0) return;
-    const long long s = r.in_off[b] + t - 1;
-    prefetch_l2(r.Ahi + s * NX * NX, (int)sizeof(float) * NX * NX);
-    prefetch_l2(r.Alo + s * NX * NX, (int)sizeof(float) * NX * NX);
-    prefetch_l2(r.Bhi + s * NX * NW, (int)sizeof(float) * NX * NW);
-    prefetch_l2(r.Blo + s * NX * NW, (int)sizeof(float) * NX * NW);
-    prefetch_l2(r.Chi + s * NY * NX, (int)sizeof(float) * NY * NX);
-    prefetch_l2(r.Clo + s * NY * NX, (int)sizeof(float) * NY * NX);
-    prefetch_l2(r.Rhi + s * NR * NR, (int)sizeof(float) * NR * NR);
-    prefetch_l2(r.Rlo + s * NR * NR, (int)sizeof(float) * NR * NR);
-    if (r.l) prefetch_l2(r.l + s * NQ, (int)sizeof(double) * NQ);
-    if (r.a) prefetch_l2(r.a + s * NX, (int)sizeof(double) * NX);
-    const long long gx = r.gs0[b] + b;
-    prefetch_l2(r.x + (gx + t) * NX, (int)sizeof(double) * 2 * NX);     // x_t, x_{t+1}
-    prefetch_l2(r.lam + (gx + t) * NX, (int)sizeof(double) * 2 * NX);   // lambda_t, lambda_{t+1}
-    prefetch_l2(r.w + r.w_off[b] + NX + (long long)(t - 1) * NW, (int)sizeof(double) * NW);
-}
-
 template <int NX, int NW, typename TR, int NY = 0>
 MHE_DEV void resid_stage(const ResidArgs<TR>& r, long long gstage, unsigned long long* sm)
 {
@@ -721,12 +967,6 @@ MHE_DEV void resid_stage(const ResidArgs<TR>& r, long long gstage, unsigned long
         resid_rows<NX, NW, 1, TR>(r, b, t, N, sm);
     } else {
         if constexpr (NY > 0) {
-            if constexpr (sizeof(TR) == 4) {
-                if (r.Ahi) {
-                    resid_mhe_df<NX, NW, NY>(r, b, t, N, sm);
-                    return;
-                }
-            }
             resid_mhe<NX, NW, NY, TR>(r, b, t, N, sm);
         } else {
             resid_q<NX, NW, TR>(r, b, t, N, sm);

@@ -31,7 +31,8 @@ constexpr int solve_words()
     using V0 = VecWs<T, NX, NW, false>;
     using V1 = VecWs<T, NX, NW, true>;
     constexpr int v = max_int(max_int(V0::rhs_count, V0::down_count), max_int(V1::rhs_count, V1::down_count));
-    constexpr int r = (v * (int)sizeof(T) + 7) / 8, q = ResidSmem<NX, NW, NY>::count;
+    constexpr int r = (v * (int)sizeof(T) + 7) / 8;
+    constexpr int q = NY > 0 ? DfWs<NX, NW, NY == 0 ? 1 : NY>::bytes / 8 : ResidSmem<NX, NW, 0>::count;
     return ((r > q ? r : q) + 1) / 2 * 2;
 }
 
@@ -68,11 +69,16 @@ MHE_DEV void instance_sync(int cluster)
 template <typename T, int NX, int NW, int NY>
 MHE_DEV void solve_residual(const ResidArgs<T>& r, int b, int N, int team, int teams, unsigned long long* sm)
 {
-    for (int t = team; t < N; t += teams) {
-        if (t == 0) resid_rows<NX, NW, 1, T>(r, b, 0, N, sm);
-        else if constexpr (NY > 0) resid_mhe_df<NX, NW, NY>(r, b, t, N, sm);
-        else resid_q<NX, NW, T>(r, b, t, N, sm);
+    if constexpr (NY > 0) {
+        StageStride it{b, team, teams, N};
+        resid_df_run<NX, NW, NY>(r, it, reinterpret_cast<unsigned char*>(sm));
         wsync();
+    } else {
+        for (int t = team; t < N; t += teams) {
+            if (t == 0) resid_rows<NX, NW, 1, T>(r, b, 0, N, sm);
+            else resid_q<NX, NW, T>(r, b, t, N, sm);
+            wsync();
+        }
     }
 }
 
