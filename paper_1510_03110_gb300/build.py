@@ -23,7 +23,7 @@ BUILD_BOUNDS = os.path.join(HERE, "_build_bounds")
 LIB_BOUNDS = os.path.join(HERE, "libmhe_bounds.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["api.cu", "engine.cpp", "plan.cpp", "shapes_small.cu", "shapes_mid.cu",
-           "shapes_big.cu", "shapes_sq.cu", "shapes_xl.cu", "shapes_xl64.cu", "shapes_n12.cu", "noalloc.cu", "serve.cu", "rts.cu", "ip.cu", "shapes_t16.cu", "shapes_t32.cu"]
+           "shapes_big.cu", "shapes_sq.cu", "shapes_xl.cu", "shapes_xl64.cu", "shapes_n12.cu", "noalloc.cu", "serve.cu", "rts.cu", "ip.cu", "shapes_t16.cu", "shapes_t32.cu", "shapes_wide.cu"]
 
 
 def nvcc() -> str:

@@ -22,6 +22,8 @@ int shapes_xl(ShapeEntry* out, int cap);
 int shapes_n12(ShapeEntry* out, int cap);
 int shapes_t16(ShapeEntry* out, int cap);
 int shapes_t32(ShapeEntry* out, int cap);
+int shapes_wide(WideEntry* out, int cap);
+int shapes_wide_small(WideEntry* out, int cap);
 int set_tc_wait_limit(int tries);   // shapes_xl.cu
 }  // namespace mhe
 
@@ -200,6 +202,19 @@ std::vector<mhe::ShapeEntry>& registry()
         // team-width variants after every default
         k += mhe::shapes_t16(buf + k, 32 - k);
         k += mhe::shapes_t32(buf + k, 32 - k);
+        // the wider reductions, beside each shape's default (its first entry)
+        mhe::WideEntry wide[16];
+        int nw = mhe::shapes_wide(wide, 16);
+        nw += mhe::shapes_wide_small(wide + nw, 16 - nw);
+        for (int w = 0; w < nw; ++w)
+            for (int i = 0; i < k; ++i)
+                if (buf[i].ops.nx == wide[w].nx && buf[i].ops.nw == wide[w].nw) {
+                    buf[i].ops.reduce64w = wide[w].reduce64;
+                    buf[i].ops.reduce32w = wide[w].reduce32;
+                    buf[i].ops.wide64 = wide[w].chunks64;
+                    buf[i].ops.wide32 = wide[w].chunks32;
+                    break;
+                }
         reg.assign(buf, buf + k);
     });
     return reg;

@@ -491,7 +491,12 @@ void Engine::reduce_level(int k, const T* A_, const T* B_, const T* Q_, const T*
     auto r32 = ops->reduce32;
     if (prec == MHE_TF32_IR && ops->reduce32tc) r32 = ops->reduce32tc;
     if (prec == MHE_BF16_IR && ops->reduce32bf) r32 = ops->reduce32bf;
-    launch<T>(ops->reduce64, r32, g, k >= 1, stream);
+    const bool tc = r32 != ops->reduce32;   // the tensor-core reductions have their own team
+    if (sizeof(T) == 8 ? (ops->reduce64w && g.nchunks <= ops->wide64)
+                       : (ops->reduce32w && !tc && g.nchunks <= ops->wide32))
+        launch<T>(ops->reduce64w, ops->reduce32w, g, k >= 1, stream);
+    else
+        launch<T>(ops->reduce64, r32, g, k >= 1, stream);
     mark(PH_REDUCE, k, 0);
 }
 

@@ -43,6 +43,10 @@ struct ShapeOps {
     long long gws64;
     int gws_teams;
     int team;   // lanes per subproblem team of these kernels
+    // the reduction with a wider team, for levels of at most wide64 / wide32 chunks (nullptr: none)
+    void (*reduce64w)(const LevelArgs<double>&, int upper, void* stream);
+    void (*reduce32w)(const LevelArgs<float>&, int upper, void* stream);
+    int wide64, wide32;
     // a whole solve with its refinement in one launch (solve.cuh), or nullptr: FP64, FP32
     // with the Q-form residual, FP32 with the double-float MHE-form residual
     void (*solve64)(const SolveArgs<double>&, void* stream);
@@ -51,6 +55,14 @@ struct ShapeOps {
     // CTAs per instance that solve takes for a batch whose longest horizon is max_N;
     // 0: one launch per level pass is the faster way
     int (*solve_cluster)(int fp64, int batch, int max_N);
+};
+
+// The reductions of one shape with wider teams (levels with few chunks).
+struct WideEntry {
+    int nx, nw;
+    void (*reduce64)(const LevelArgs<double>&, int upper, void* stream);
+    void (*reduce32)(const LevelArgs<float>&, int upper, void* stream);
+    int chunks64, chunks32;   // the most chunks of a level the wider team is the faster one for
 };
 
 // Everything one compiled shape provides (one entry per shape and team width).

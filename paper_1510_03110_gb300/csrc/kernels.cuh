@@ -24,10 +24,15 @@ enum { OP_REDUCE = 0, OP_RHS = 1, OP_DOWN = 2, OP_REDUCE_TC = 3, OP_REDUCE_BF = 
 // the mbarrier and the TMEM address
 constexpr int kTcExtra = 8192 + 4;
 
+// shapes whose reduction runs reduce_chunk_small (pivot blocks of at most 32 rows)
+template <int NX>
+constexpr bool small_shape() { return NX <= 32; }
+
 // shared-memory workspace (elements of T) one team of a pass needs
 template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int op_count()
 {
+    if (OP == OP_REDUCE && small_shape<NX>()) return RedWs<T, NX, NW, UPPER != 0>::count;
     return (OP == OP_REDUCE || OP == OP_DOWN_LIT)
                ? Ws<T, NX>::count
                : (OP == OP_RHS ? VecWs<T, NX, NW, UPPER != 0>::rhs_count
@@ -56,10 +61,26 @@ constexpr int op_max_teams()
     return vector_op<OP>() ? (MHE_TEAM >= 128 ? 1 : 128 / MHE_TEAM) : kMaxTeams;
 }
 
+// CTAs of w teams of `bytes` each that fit an SM (228 KB, of which a CTA takes 1 KB beside its own)
+constexpr int ctas_per_sm(int w, int bytes) { return 228 * 1024 / (w * bytes + 1024); }
+// teams per CTA that leave the least shared memory unused, whole warps, at most 256 threads
+constexpr int best_teams(int bytes)
+{
+    const int step = MHE_TEAM >= 32 ? 1 : 32 / MHE_TEAM;
+    int best = step, most = 0;
+    for (int w = step; w <= kMaxTeams; w += step) {
+        if (w * bytes > kLevelSmem) break;
+        const int n = w * ctas_per_sm(w, bytes);
+        if (n > most || (n == most && w * MHE_TEAM <= 128)) { most = n; best = w; }
+    }
+    return best;
+}
+
 // teams per CTA: as many per-team workspaces as fit in kLevelSmem, at most the op's
 template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int level_warps()
 {
+    if (OP == OP_REDUCE && small_shape<NX>()) return best_teams((int)(op_count<T, NX, NW, UPPER, OP>() * sizeof(T)));
     constexpr int fit = kLevelSmem / (int)(op_count<T, NX, NW, UPPER, OP>() * sizeof(T));
     return fit >= op_max_teams<OP>() ? op_max_teams<OP>() : (fit < 1 ? 1 : fit);
 }
@@ -69,6 +90,12 @@ template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr bool level_fits()
 {
     return (long long)op_count<T, NX, NW, UPPER, OP>() * (long long)sizeof(T) <= 227LL * 1024;
+}
+
+template <typename T, int NX, int NW, int UPPER, int OP>
+constexpr int level_threads()
+{
+    return vector_op<OP>() ? 128 : (OP == OP_REDUCE && small_shape<NX>() ? level_warps<T, NX, NW, UPPER, OP>() * MHE_TEAM : 256);
 }
 
 // CTAs of 256 threads per SM the register allocation is sized for: the small
@@ -87,6 +114,13 @@ constexpr int level_min_blocks()
         constexpr int bytes = level_warps<T, NX, NW, UPPER, OP>() * op_count<T, NX, NW, UPPER, OP>() * (int)sizeof(T);
         constexpr int fit = 228 * 1024 / (bytes + 1024);
         return fit > 8 ? 8 : (fit < 1 ? 1 : fit);
+    }
+    if (OP == OP_REDUCE && small_shape<NX>()) {
+        // what shared memory holds, with at least 96 registers a thread
+        constexpr int w = level_warps<T, NX, NW, UPPER, OP>();
+        constexpr int fit = ctas_per_sm(w, op_count<T, NX, NW, UPPER, OP>() * (int)sizeof(T));
+        constexpr int regs = 65536 / (w * MHE_TEAM * 96);
+        return fit < regs ? (fit < 1 ? 1 : fit) : (regs < 1 ? 1 : regs);
     }
     return NX >= 48 ? 1   // four-warp teams, a few per SM: every pass may take 255 registers
                     : (sizeof(T) == 4
@@ -113,7 +147,7 @@ constexpr bool tc_shape()
 constexpr int kGwsTeams = 2 * 152;
 
 template <typename T, int NX, int NW, int UPPER, int OP>
-__global__ void __launch_bounds__(vector_op<OP>() ? 128 : 256, level_min_blocks<T, NX, NW, UPPER, OP>()) k_level(LevelArgs<T> a)
+__global__ void __launch_bounds__(level_threads<T, NX, NW, UPPER, OP>(), level_min_blocks<T, NX, NW, UPPER, OP>()) k_level(LevelArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int W = level_warps<T, NX, NW, UPPER, OP>();
@@ -159,6 +193,8 @@ __global__ void __launch_bounds__(vector_op<OP>() ? 128 : 256, level_min_blocks<
         if (threadIdx.x < 32) tc::tmem_dealloc(tcs.tbase, 512);
     } else if (!chunk_in_bounds(a, ci)) {
         return;
+    } else if constexpr (OP == OP_REDUCE && small_shape<NX>()) {
+        reduce_chunk_small<T, NX, NW, UPPER != 0>(a, ci, sm);
     } else if (OP == OP_REDUCE) {
         reduce_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
     } else if (OP == OP_RHS) {
@@ -406,6 +442,9 @@ ShapeEntry make_shape()
     e.ops.resid_mhe32 = &launch_resid<NX, NW, float, NY>;
     e.ops.gws64 = 0;
     e.ops.gws_teams = 0;
+    e.ops.reduce64w = nullptr;
+    e.ops.reduce32w = nullptr;
+    e.ops.wide64 = e.ops.wide32 = 0;
     if constexpr (NX <= 32) {
         e.ops.solve64 = &launch_solve<double, NX, NW, 0>;
         e.ops.solve32 = &launch_solve<float, NX, NW, 0>;
@@ -419,6 +458,23 @@ ShapeEntry make_shape()
     e.ny = NY;
     e.assemble = &launch_assemble<NX, NW, NY>;
     return e;
+}
+
+// A level's reduction with this unit's wider team.  Up to how many chunks it pays, from both sides measured
+// on GB300: FP64 nx = 20, 512 leaf chunks 2.37 -> 2.04 ms (32 -> 128 lanes), 128 master chunks 0.58 -> 0.22 ms; FP64
+// nx = 12, 316 chunks 0.29 -> 0.14 ms, 1125 chunks 0.36 -> 0.33 ms (16 -> 128 lanes); FP32 nx = 24, 362 chunks 41 -> 33
+// us, 1201 chunks 170 -> 175 us.
+template <int NX, int NW>
+WideEntry make_wide()
+{
+    WideEntry w;
+    w.nx = NX;
+    w.nw = NW;
+    w.reduce64 = &launch_level<double, NX, NW, OP_REDUCE>;
+    w.reduce32 = &launch_level<float, NX, NW, OP_REDUCE>;
+    w.chunks64 = NX <= 12 && MHE_TEAM == 128 ? 1216 : 608;
+    w.chunks32 = 608;
+    return w;
 }
 
 // The FP64 passes of a shape whose FP64 reduction workspace exceeds an SM's

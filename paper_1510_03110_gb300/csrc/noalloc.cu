@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(32) k_serial_noalloc(int N, const double* A, c
     g.piv_rel = 1e-14;
     g.store_P = 0;
     double* sm = reinterpret_cast<double*>(smem_raw);
-    mhe::reduce_chunk<double, NX, NW, false>(g, 0, sm);
+    mhe::reduce_chunk_small<double, NX, NW, false>(g, 0, sm);
     g.xd = x; g.wd = w; g.ld = lam;
     mhe::down_chunk<double, NX, NW, false>(g, 0, sm);
     __syncwarp();
@@ -98,7 +98,7 @@ struct Entry {
 template <int NX, int NW>
 Entry entry()
 {
-    constexpr int c = mhe::max_int(mhe::Ws<double, NX>::count, mhe::VecWs<double, NX, NW, false>::down_count);
+    constexpr int c = mhe::max_int(mhe::RedWs<double, NX, NW, false>::count, mhe::VecWs<double, NX, NW, false>::down_count);
     return Entry{NX, NW, &k_serial_noalloc<NX, NW>, c * sizeof(double)};
 }
 

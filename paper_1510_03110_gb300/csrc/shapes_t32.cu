@@ -14,4 +14,13 @@ int shapes_t32(ShapeEntry* out, int cap)
     return k;
 }
 
+// the reductions of the smallest shapes with a warp per subproblem, for levels with few chunks
+int shapes_wide_small(WideEntry* out, int cap)
+{
+    int k = 0;
+    if (k < cap) out[k++] = make_wide<4, 2>();
+    if (k < cap) out[k++] = make_wide<6, 3>();
+    return k;
+}
+
 }  // namespace mhe

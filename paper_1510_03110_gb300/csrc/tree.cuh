@@ -30,6 +30,7 @@
 
 #include "common.h"
 #include "f32conv.h"
+#include "reduce.cuh"
 #include "stage.cuh"
 #include "tc.cuh"
 #include "vec.cuh"
@@ -198,73 +199,6 @@ MHE_DEV bool chol_inplace(Ws<T, NX>& s, T* Gm, double piv_rel)
         });
     }
     return s.sc[1] != 0;
-}
-
-// Rank-revealing (pivoted) Cholesky of the symmetric NX x NX matrix Gm (both
-// triangles held): at step j the largest remaining diagonal is brought to (j, j)
-// by a symmetric row and column swap; the factorisation stops at the first step
-// whose largest remaining diagonal is at or below rank_rel * max diag, and that
-// step is the numerical rank r.  On return Pi^T Gm_in Pi = L L^T restricted to
-// r columns: L (lower trapezoidal, NX x r) in Gm's lower part, the pivot order
-// Pi in permv (as values of T), and r is returned.
-template <typename T, int NX>
-MHE_DEV int chol_pivoted(Ws<T, NX>& s, T* Gm, double rank_rel, T* permv)
-{
-    constexpr int ld = Ws<T, NX>::ld;
-    wone([&](int) {
-        T mx = 0;
-        for (int i = 0; i < NX; ++i) {
-            mx = mmax(mx, mabs(Gm[i + i * ld]));
-            permv[i] = (T)i;
-        }
-        s.sc[0] = (T)(rank_rel * (double)mx);
-        s.sc[3] = (T)NX;
-    });
-    for (int j = 0; j < NX; ++j) {
-        wone([&](int) {
-            int p = j;
-            T best = Gm[j + j * ld];
-            for (int i = j + 1; i < NX; ++i)
-                if (Gm[i + i * ld] > best) { best = Gm[i + i * ld]; p = i; }
-            s.sc[4] = (T)p;
-            if (!(best > s.sc[0])) s.sc[3] = (T)j;   // the rank: nothing above the threshold remains
-        });
-        if ((int)s.sc[3] == j) break;   // the same value for every lane (read after the barrier)
-        const int p = (int)s.sc[4];
-        if (p != j) {
-            wfor(NX, [&](int q) {
-                const T t = Gm[j + q * ld];
-                Gm[j + q * ld] = Gm[p + q * ld];
-                Gm[p + q * ld] = t;
-            });
-            wfor(NX, [&](int q) {
-                const T t = Gm[q + j * ld];
-                Gm[q + j * ld] = Gm[q + p * ld];
-                Gm[q + p * ld] = t;
-            });
-            wone([&](int) {
-                const T t = permv[j];
-                permv[j] = permv[p];
-                permv[p] = t;
-            });
-        }
-        wone([&](int) {
-            const T l = msqrt(Gm[j + j * ld]);
-            Gm[j + j * ld] = l;
-            s.sc[2] = l;
-        });
-        const T ljj = s.sc[2];
-        wfor(NX, [&](int i) {
-            if (i > j) Gm[i + j * ld] /= ljj;
-        });
-        // the trailing block, both triangles (the next pivot search and swaps read them)
-        const int rem = NX - j - 1;
-        wfor(rem * rem, [&](int u) {
-            const int i = j + 1 + u % rem, c = j + 1 + u / rem;
-            Gm[i + c * ld] -= Gm[i + j * ld] * Gm[c + j * ld];
-        });
-    }
-    return (int)s.sc[3];
 }
 
 template <typename T, int NX, int MT>
@@ -947,7 +881,7 @@ MHE_DEV void reduce_chunk(const LevelArgs<T>& a, int ci, T* smem, TcState* tcs =
         // recovers w^ = Pi [L_11^{-T} w^'_{1..r}; 0].
         int rank = NX;
         if (a.piv_up) {
-            rank = chol_pivoted<T, NX>(s, s.Qw, a.piv_rank, s.u);
+            rank = chol_pivoted<T, NX, ld>(s.Qw, a.piv_rank, s.u, s.sc);
             if (rank == 0 && bad_t < 0) bad_t = cd.t0;
         } else if (chol_inplace<T, NX, NX>(s, s.Qw, a.piv_rel) && bad_t < 0) {
             bad_t = cd.t0;
