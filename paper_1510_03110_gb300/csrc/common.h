@@ -145,6 +145,7 @@ struct SolveArgs {
     int batch, nlev;
     int cluster;                       // CTAs per instance
     int fused_rhs;                     // the factorisation ran the vector part: start with the down pass
+    int resume;                        // continue with the next correction of the instances still active
     int max_refine;
     double tol;
     // per level: the pass with the problem's right-hand side, and the corrections' pass

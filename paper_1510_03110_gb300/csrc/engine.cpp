@@ -691,21 +691,34 @@ void launch_solve(const ShapeOps* ops, const SolveArgs<float>& p, void* s)
 }
 }  // namespace
 
+namespace {
+constexpr int kPassRounds = 4;   // corrections launched pass by pass before the rest goes to one launch
+}
+
 // A batch of few or small instances is bound by launches and by the latency of the small upper
 // levels: one launch takes the vector pass, the down pass and every correction of an instance in
 // a cluster of its own, which stops when the instance has converged.  Timing marks want a launch
 // per level pass; FP64 master levels, the literal down pass and the FP64-instruction MHE residual
 // have no fused form.
+//
+// resume: a larger batch's last corrections.  Its passes are launched one by one for the first kPassRounds
+// corrections; what is left then is usually nothing or a few instances, and the corrections still allowed
+// would cost a dozen launches each: one launch takes them, whose clusters without work return at once.
+bool Engine::has_fused(bool fp64) const
+{
+    if (!ops->solve_cluster || !ordered || m64 || literal || mark_user || lv.size() > (size_t)kSolveLevels) return false;
+    if (mheC && (fp64 || !rAh)) return false;
+    return fp64 ? ops->solve64 != nullptr : (mheC ? ops->solve_mhe32 != nullptr : ops->solve32 != nullptr);
+}
+
 template <typename T>
 bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
-                         bool fused)
+                         bool fused, bool resume)
 {
     const bool fp64 = sizeof(T) == 8;
     const size_t L = lv.size();
-    if (!ops->solve_cluster || !ordered || m64 || literal || mark_user || L > (size_t)kSolveLevels) return false;
-    if (mheC && (fp64 || !rAh)) return false;
-    if (fp64 ? !ops->solve64 : (mheC ? !ops->solve_mhe32 : !ops->solve32)) return false;
-    const int cl = ops->solve_cluster(fp64, plan.batch, plan.max_N);
+    if (!has_fused(fp64)) return false;
+    const int cl = resume ? 4 : ops->solve_cluster(fp64, plan.batch, plan.max_N);
     if (cl < 1) return false;
     SolveArgs<T> p;
     memset(&p, 0, sizeof(p));
@@ -713,6 +726,7 @@ bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0
     p.nlev = (int)L;
     p.cluster = cl;
     p.fused_rhs = fused;
+    p.resume = resume;
     p.max_refine = max_refine;
     p.tol = tol;
     T* d[3] = {static_cast<T*>(dx), static_cast<T*>(dw), static_cast<T*>(dl)};
@@ -732,7 +746,7 @@ bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0
     p.iters = iters;
     p.active = active;
     p.info = reinterpret_cast<mhe_info_rec*>(info_dev);
-    if (!fp64) { p.zx = x; p.zw = w; p.zl = lam; }
+    if (!fp64 && !resume) { p.zx = x; p.zw = w; p.zl = lam; }
     ++launches;
     launch_solve(ops, p, stream);
     return true;
@@ -769,6 +783,7 @@ int Engine::run_solve(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, d
     const T* cra0 = static_cast<const T*>(ra0);
     const T* crlN = static_cast<const T*>(rlN);
     const T* crx0 = static_cast<const T*>(rx0);
+    bool resumed = false;
     for (int it = 0; it < max_refine; ++it) {
         any_mask = it == 0 ? nullptr : any_act;
         residual<T>(rhs, x, w, lam, it == 0 ? nullptr : active);
@@ -777,6 +792,10 @@ int Engine::run_solve(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, d
                      any_act, dznorm, stream);
         ++launches;
         any_mask = any_act;
+        if (it == kPassRounds && solve_fused<T>(rhs, l, a, x0, x, w, lam, false, true)) {
+            resumed = true;
+            break;
+        }
         if (m64) {   // the correction's x~0 for the FP64 master levels
             rt->widen(rx0_64, static_cast<const float*>(rx0), (long long)plan.batch * plan.n, stream);
             ++launches;
@@ -793,8 +812,9 @@ int Engine::run_solve(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, d
     }
     // final check: after a refinement loop only the instances corrected since
     // their last residual (still active) need one
+    // (the fused launch has checked its own, and left none active)
     any_mask = max_refine > 0 ? any_act : nullptr;
-    residual<T>(rhs, x, w, lam, max_refine > 0 ? active : nullptr);
+    if (!resumed) residual<T>(rhs, x, w, lam, max_refine > 0 ? active : nullptr);
     any_mask = nullptr;
     rt->finalize(plan.batch, norms, kinf, active, iters, status, where, tol, 2, max_refine > 0 ? 3 : 0, info_dev,
                  nullptr, dznorm, stream);

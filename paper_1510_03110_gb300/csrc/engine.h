@@ -260,7 +260,8 @@ private:
     // the solve and its refinement in one launch, when the shape and the batch suit it
     template <typename T>
     bool solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0, double* x, double* w, double* lam,
-                     bool fused);
+                     bool fused, bool resume = false);
+    bool has_fused(bool fp64) const;
     template <typename T>
     ResidArgs<T> resid_args(const mhe_rhs* rhs, const double* x, const double* w, const double* lam) const;
     template <typename T>

@@ -16,8 +16,14 @@
 // What bounds it.  FP64: an instruction of a warp costs 64 cycles of its SM quarter whatever
 // its number of active lanes, so the products are dealt to lanes entry by entry (no
 // lane tile whose corners stick out) and only one triangle of the symmetric ones is formed.
-// FP32: the latency of the chain at eight to sixteen warps an SM; the products use
-// register tiles (TM + TN shared-memory loads per TM TN FMAs).
+// FP32: the latency of the chain at ten to twenty warps an SM, and the shared-memory loads of the products (register
+// tiles, TM + TN loads of 16 bytes per 2 TM TN packed FMAs; ncu at nx = 24: 35% issue, 54% of the shared-memory
+// wavefronts).
+//
+// Measured (GB300), before (some twenty barriers a stage, both triangles, divisions, blocks loaded as the
+// stage came) and after: FP64 nx = 20, 16384 stages in chunks of 32, 3.75 -> 2.04 ms, with four warps a chunk; a
+// master level of it 0.92 -> 0.22 ms; FP32 leaf level nx = 6, 1.10M stages, 1.02 -> 0.55 ms; nx = 12, 1.05M stages, 2.65 -> 2.08
+// ms; nx = 24, 535k stages, 6.44 -> 5.85 ms.
 #pragma once
 #include <type_traits>
 
@@ -64,6 +70,14 @@ constexpr int prod_tile(int M, int N, int LN, bool sym)
     return best;
 }
 
+MHE_DEV void ldp(const float* p, F2 (&v)[2])
+{
+    const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = q.x;
+    v[1] = q.y;
+}
+MHE_DEV void ldp(const float* p, F2 (&v)[1]) { v[0] = *reinterpret_cast<const F2*>(p); }
+
 // out(i, j, sum_p A[p + i LDA] B[p + j LDB] , q) for i < M, j < N (SYM: the pairs of a symmetric result, each
 // once, in either order), on the lanes L0 .. L0 + LN - 1 of the team, no barrier.
 // pre(i, j) is loaded before the sum and handed to out.  Both operands are read by columns in vectors.
@@ -97,23 +111,53 @@ MHE_DEV void prod(const T* A, const T* B, FP&& pre, FO&& out)
                 if ((M % TM == 0 || i < M) && (N % TN == 0 || j < N)) pv[r][c] = pre(i, j);
             }
         T acc[TM][TN];
+        if constexpr (sizeof(T) == 4 && VA >= 2) {
+            // the even and the odd terms side by side: pairs as they lie in memory, half the instructions
+            F2 s[TM][TN];
 #pragma unroll
-        for (int r = 0; r < TM; ++r)
+            for (int r = 0; r < TM; ++r)
 #pragma unroll
-            for (int c = 0; c < TN; ++c) acc[r][c] = (T)0;
+                for (int c = 0; c < TN; ++c) s[r][c] = 0ULL;
+#pragma unroll(TM * TN >= 9 ? 3 : 6)
+            for (int p = 0; p < K; p += VA) {
+                F2 av[TM][VA / 2], bv[TN][VA / 2];
+#pragma unroll
+                for (int r = 0; r < TM; ++r) ldp(ap[r] + p, av[r]);
+#pragma unroll
+                for (int c = 0; c < TN; ++c) ldp(bp[c] + p, bv[c]);
+#pragma unroll
+                for (int q = 0; q < VA / 2; ++q)
+#pragma unroll
+                    for (int r = 0; r < TM; ++r)
+#pragma unroll
+                        for (int c = 0; c < TN; ++c) s[r][c] = fma2(av[r][q], bv[c][q], s[r][c]);
+            }
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+#pragma unroll
+                for (int c = 0; c < TN; ++c) {
+                    const float2 v = unpack2(s[r][c]);
+                    acc[r][c] = v.x + v.y;
+                }
+        } else {
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+#pragma unroll
+                for (int c = 0; c < TN; ++c) acc[r][c] = (T)0;
 #pragma unroll(sizeof(T) == 8 ? K / VA : (TM * TN >= 9 ? 3 : 6))
-        for (int p = 0; p < K; p += VA) {
-            T av[TM][VA], bv[TN][VA];
+            for (int p = 0; p < K; p += VA) {
+                T av[TM][VA], bv[TN][VA];
 #pragma unroll
-            for (int r = 0; r < TM; ++r) ldv(ap[r] + p, av[r]);
+                for (int r = 0; r < TM; ++r) ldv(ap[r] + p, av[r]);
 #pragma unroll
-            for (int c = 0; c < TN; ++c) ldv(bp[c] + p, bv[c]);
+                for (int c = 0; c < TN; ++c) ldv(bp[c] + p, bv[c]);
 #pragma unroll
-            for (int q = 0; q < VA; ++q)
+                for (int q = 0; q < VA; ++q)
 #pragma unroll
-                for (int r = 0; r < TM; ++r)
+                    for (int r = 0; r < TM; ++r)
 #pragma unroll
-                    for (int c = 0; c < TN; ++c) acc[r][c] += av[r][q] * bv[c][q];
+                        for (int c = 0; c < TN; ++c) acc[r][c] += av[r][q] * bv[c][q];
+            }
         }
 #pragma unroll
         for (int r = 0; r < TM; ++r)
@@ -502,24 +546,36 @@ MHE_DEV bool reduce_stage(RedPtr<T>& s, const StageRef<T>& st, T* Pout, T* Lgout
             });
         wsync();
         // 2. the blocks of W^T P W + Q:  F -> P,  H^T -> Y,  G;  A^T u -> t,  g = B^T u - l_w -> Y's last column
-        prod<T, NX + MT, NX + MT, NX, ld, ld, true, 0, TL>(
-            s.W, s.X, [&](int i, int j) -> T { return i <= j ? X::q(st, i, j) : X::q(st, j, i); },
-            [&](int i, int j, T v, T q) {
-                v += q;
-                if (i > j) {
-                    const int k = i;
-                    i = j;
-                    j = k;
-                }
-                if (j < NX) {
-                    s.P[i + j * ld] = v;
-                    s.P[j + i * ld] = v;
-                } else if (i < NX) {
-                    s.Y[(j - NX) + i * lm] = v;
-                } else {
-                    s.G[(j - NX) + (i - NX) * lm] = v;
-                }
-            });
+        if constexpr (sizeof(T) == 8 || NX < 16) {   // all blocks dealt out together: the fewest rounds
+            prod<T, NX + MT, NX + MT, NX, ld, ld, true, 0, TL>(
+                s.W, s.X, [&](int i, int j) -> T { return i <= j ? X::q(st, i, j) : X::q(st, j, i); },
+                [&](int i, int j, T v, T q) {
+                    v += q;
+                    if (i > j) {
+                        const int k = i;
+                        i = j;
+                        j = k;
+                    }
+                    if (j < NX) {
+                        s.P[i + j * ld] = v;
+                        s.P[j + i * ld] = v;
+                    } else if (i < NX) {
+                        s.Y[(j - NX) + i * lm] = v;
+                    } else {
+                        s.G[(j - NX) + (i - NX) * lm] = v;
+                    }
+                });
+        } else {
+            prod<T, NX, NX, NX, ld, ld, true, 0, TL>(
+                s.W, s.X, [&](int i, int j) -> T { return X::qx(st, i, j); },
+                [&](int i, int j, T v, T q) { s.P[i + j * ld] = s.P[j + i * ld] = v + q; });
+            prod<T, NX, MT, NX, ld, ld, false, 0, TL>(
+                s.W, s.X + ld * NX, [&](int i, int j) -> T { return X::qxw(st, i, j); },
+                [&](int i, int j, T v, T q) { s.Y[j + i * lm] = v + q; });
+            prod<T, MT, MT, NX, ld, ld, true, 0, TL>(
+                s.W + ld * NX, s.X + ld * NX, [&](int i, int j) -> T { return X::qw(st, i, j); },
+                [&](int i, int j, T v, T q) { s.G[i + j * lm] = s.G[j + i * lm] = v + q; });
+        }
         each<NX + MT>([&](int i) {
             const T d = coldot<NX>(s.W + i * ld, u, (T)0);
             if (i < NX) s.t[i] = d;

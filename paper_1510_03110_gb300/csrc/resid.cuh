@@ -359,39 +359,8 @@ MHE_DEV float2 df_split(double v)
     return make_float2(h, f32_lo(v, h));
 }
 
-// Two double-float accumulators side by side in packed FP32 instructions (fma.rn.f32x2 and the
-// like work on register pairs): the even and the odd terms of a dot product, half the issue slots.
-using F2 = unsigned long long;
-MHE_DEV F2 pack2(float x, float y)
-{
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-MHE_DEV float2 unpack2(F2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-MHE_DEV F2 fma2(F2 a, F2 b, F2 c)
-{
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-MHE_DEV F2 add2(F2 a, F2 b)
-{
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-MHE_DEV F2 mul2(F2 a, F2 b)
-{
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
+// Two double-float accumulators side by side in packed FP32 instructions: the even and the odd
+// terms of a dot product, half the issue slots.
 MHE_DEV F2 sub2(F2 a, F2 b) { return fma2(b, pack2(-1.f, -1.f), a); }   // exact product: one rounding, as a - b
 
 // the sums s and their compensations: rounding errors of the sums (c) and the products' parts (d)

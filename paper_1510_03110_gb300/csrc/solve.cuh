@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(solve_threads<T, NX, NW, NY>(), 2) k_solve(con
     unsigned long long* sm =
         reinterpret_cast<unsigned long long*>(smem_raw) + (size_t)team_id() * solve_words<T, NX, NW, NY>();
     T* ws = reinterpret_cast<T*>(sm);
+    if (p.resume && !p.active[b]) return;   // the whole cluster
     const LevelInst li = p.lv[0].li[b];
     const int N = li.N;
     unsigned long long* norms = p.r.norms + 3LL * b;
@@ -109,9 +110,10 @@ __global__ void __launch_bounds__(solve_threads<T, NX, NW, NY>(), 2) k_solve(con
         norms[0] = norms[1] = norms[2] = 0ULL;
         p.dznorm[b] = 0u;
     }
-    int iters = 0;
+    // resumed: the check that left the instance active counted the correction that comes now
+    int iters = p.resume ? p.iters[b] : 0;
     double relres = 0.0, est = 0.0;
-    for (int it = -1;; ++it) {
+    for (int it = p.resume ? 0 : -1;; ++it) {
         const int v0 = it < 0 ? 0 : kSolveLevels;
         if (it >= 0 || !p.fused_rhs) {
 #pragma unroll 1
@@ -176,6 +178,7 @@ __global__ void __launch_bounds__(solve_threads<T, NX, NW, NY>(), 2) k_solve(con
         o.est_relerr = est;
         p.info[b] = o;
         p.iters[b] = iters;
+        p.active[b] = 0;
     }
 }
 

@@ -83,6 +83,40 @@ MHE_DEV void async_vec(T* dst, const T* src)
         for (int i = lane_id(); i < N; i += MHE_TEAM) dst[i] = (T)0;
 }
 
+// ---- packed FP32 pairs (fma.rn.f32x2 and the like work on register pairs) ------
+
+using F2 = unsigned long long;
+MHE_DEV F2 pack2(float x, float y)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+MHE_DEV float2 unpack2(F2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+MHE_DEV F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+MHE_DEV F2 add2(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+MHE_DEV F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // ---- products with shared-memory operands -------------------------------------
 
 // the widest vector (16 or 8 bytes, else one entry) whole columns of n entries can be read in
