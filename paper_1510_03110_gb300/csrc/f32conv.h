@@ -104,4 +104,39 @@ MHE_HD float f32_lo(double d, float hi)
     return f32_lo_rare(d, hi);
 }
 
+// hi = f32_rn(v) and lo = f32_lo(v, hi) with the work they share done once (the conversions are most of
+// the preparation pass's instructions: about twenty here, about forty by the two functions).
+MHE_HD void f32_pair(double v, float& hi, float& lo)
+{
+    unsigned long long u;
+    memcpy(&u, &v, sizeof(u));
+    const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
+    const unsigned sign = uh & 0x80000000u, e = (uh >> 20) & 0x7FFu;
+    if (e - 949u <= 201u) {   // a normal float whose rest has a normal scale
+        // the high word shifted left by three holds the top 23 fraction bits and the low eight exponent bits;
+        // e - 896 differs from those in the top one
+        const unsigned f = (((uh << 3) | (ul >> 29)) & 0x7FFFFFFFu) ^ 0x40000000u;
+        const unsigned rem = ul & 0x1FFFFFFFu;
+        const unsigned up = rem + (f & 1u) > 0x10000000u ? 1u : 0u;   // to nearest, ties to even
+        const int r = (int)(rem - (up << 29));
+#ifdef __CUDA_ARCH__
+        const float fr = __int2float_rn(r);
+#else
+        const float fr = (float)r;
+#endif
+        const unsigned sb = (f & 0x7F800000u) - (52u << 23);   // 2^(e - 1075)
+        float scale;
+        memcpy(&scale, &sb, sizeof(scale));
+        const float rest = fr * scale;
+        unsigned hb = (f + up) | sign, lb;
+        memcpy(&lb, &rest, sizeof(lb));
+        lb ^= sign;
+        memcpy(&hi, &hb, sizeof(hi));
+        memcpy(&lo, &lb, sizeof(lo));
+        return;
+    }
+    hi = f32_rn(v);
+    lo = f32_lo(v, hi);
+}
+
 }  // namespace mhe

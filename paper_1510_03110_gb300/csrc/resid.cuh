@@ -13,6 +13,7 @@
 #pragma once
 #include "common.h"
 #include "f32conv.h"
+#include "reduce.cuh"
 #include "vec.cuh"
 #include "warp.cuh"
 #include "wgemm.cuh"
@@ -1089,41 +1090,73 @@ MHE_DEV void assemble_stage(const double* C, const double* R, const double* yt, 
 // FP64 dot products of l dealt to lanes without branch divergence.
 template <int NX, int NW, int NY>
 struct PrepSmem {
-    static constexpr int NR = NW + NY;
-    // odd leading dimensions: the lanes of a product tile or a row sum read
-    // down a column or along a row of these blocks without bank conflicts
-    static constexpr int odd(int n) { return n | 1; }
-    static constexpr int LC = odd(NY), LR = odd(NR), LA = odd(NX), LS = odd(NW);
+    static constexpr int NR = NW + NY, NQ = NX + NW;
     static constexpr int nd = NY + NW + NY;   // doubles: y~, w~, t = S^T w~ - V y~
-    // floats: C, R, A (later Q_x), B (later V C), S C, row sums
-    static constexpr int nb = LA * NW > LC * NX ? LA * NW : LC * NX;
-    static constexpr int nf = LC * NX + LR * NR + LA * NX + nb + LS * NX + 2 * NX + NW + 1;
-    static constexpr int count = nd + (nf + 1) / 2;   // 8-byte words
+    // floats: C and V C by columns, R by rows (its rows are the products' contiguous operand); A and B
+    // (odd leading dimension: read along rows and columns) for their row sums, then Q in their place
+    static constexpr int ldC = pick_ld(NY, vec_of<float>(NY)), ldR = pick_ld(NR, vec_of<float>(NR)), ldA = NX | 1;
+    static constexpr int oC = round_to(nd, 2) * 2, oVC = oC + round_to(ldC * NX, 4), oR = oVC + round_to(ldC * NX, 4),
+                         oQ = oR + round_to(ldR * NR, 4), oB = oQ + ldA * NX;
+    static constexpr int nq = max_int(NQ * NQ, ldA * NQ);
+    static constexpr int count = (oQ + round_to(nq, 4)) / 2;   // 8-byte words
+    static_assert(NW % vec_of<float>(NY) == 0, "the S and V parts of a row of R start on a whole vector");
 };
+
+// f(i, src[i]) for i < COUNT, lanes round-robin, the next eight loads of a lane in flight while it works on eight.
+// The rounds are not unrolled: a preparation stage unrolled in full outgrows the instruction cache (at nx = 64
+// ten of thirteen warp cycles per instruction went into waiting for instructions).
+template <int COUNT, class F>
+MHE_DEV void stream_in(const double* src, F&& f)
+{
+    constexpr int PER = (COUNT + MHE_TEAM - 1) / MHE_TEAM, CH = PER < 6 ? PER : 6, NB = (PER + CH - 1) / CH;
+    double cur[CH], nxt[CH];
+    auto load = [&](double (&v)[CH], int k0) {
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            const int i = lane_id() + MHE_TEAM * (k0 + k);
+            v[k] = i < COUNT ? src[i] : 0.0;
+        }
+    };
+    load(cur, 0);
+#pragma unroll 1
+    for (int c = 0; c < NB; ++c) {
+        if (c + 1 < NB) load(nxt, (c + 1) * CH);
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            const int i = lane_id() + MHE_TEAM * (c * CH + k);
+            if (i < COUNT) f(i, cur[k]);
+            cur[k] = nxt[k];
+        }
+    }
+}
 
 template <int NX, int NW, int NY>
 MHE_DEV void prep_stage(const PrepArgs& p, long long gstage, double* sm)
 {
     using PS = PrepSmem<NX, NW, NY>;
     constexpr int NR = NW + NY, NQ = NX + NW;
-    constexpr int LC = PS::LC, LR = PS::LR, LA = PS::LA, LS = PS::LS;
+    constexpr int ldC = PS::ldC, ldR = PS::ldR, ldA = PS::ldA;
     const int b = stage_instance(p.gs0, p.batch, gstage);
     const int t = (int)(gstage - p.gs0[b]);
     double* dy = sm;
     double* dw = dy + NY;
     double* dt = dw + NW;
-    // A and B are only read for the row sums of ||K||_inf, taken right after the
-    // load; Q_x and V C then reuse their space (fewer bytes per team, more teams per SM).
-    // Blocks column-major with the padded leading dimensions LC (C, V C), LR (R),
-    // LA (A, Q_x, B), LS (S C).
-    float* fC = reinterpret_cast<float*>(sm + PS::nd);
-    float* fR = fC + LC * NX;
-    float* fA = fR + LR * NR;
-    float* fQx = fA;
-    float* fB = fA + LA * NX;
-    float* fVC = fB;
-    float* fSC = fB + PS::nb;
-    float* rsum = fSC + LS * NX;
+    float* sf = reinterpret_cast<float*>(sm);
+    float *fC = sf + PS::oC, *fVC = sf + PS::oVC, *fR = sf + PS::oR, *fQ = sf + PS::oQ;
+    float *fA = fQ, *fB = sf + PS::oB;
+    // the largest row sum of this lane, merged over the team into the instance's ||K||_inf
+    auto merge = [&](float m) {
+        constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32;
+        const unsigned mask =
+            CW == 32 ? 0xffffffffu : (((1u << CW) - 1u) << ((threadIdx.x & 31) & ~(CW - 1)));
+        unsigned u = float_bits(m);
+#pragma unroll
+        for (int d = CW / 2; d > 0; d /= 2) {
+            const unsigned o = __shfl_xor_sync(mask, u, d, CW);
+            u = o > u ? o : u;
+        }
+        if ((lane_id() & (CW - 1)) == 0) atomic_max_u32(p.kinf + b, u);
+    };
     if (t == 0) {
         // arrival stage: x rows 1 + 1, w rows |P~0^{-1} row| + 1, dynamics rows 3, initial row 1
         const double* P0 = p.P0inv + (long long)b * NX * NX;
@@ -1131,109 +1164,72 @@ MHE_DEV void prep_stage(const PrepArgs& p, long long gstage, double* sm)
         wcopy<NX * NX>([&](int i) { return P0[i]; }, [&](int i, double v) {
             const float f = f32_rn(v);
             P0f[i] = f;
-            fA[i % NX + (i / NX) * LA] = f;
+            fA[i % NX + (i / NX) * ldA] = f;
         });
-        wfor(NX, [&](int i) {
+        float m = 3.f;
+        each<NX>([&](int i) {
             p.x0_32[(long long)b * NX + i] = f32_rn(p.x0[(long long)b * NX + i]);
             float rs = 1.f;
-            for (int j = 0; j < NX; ++j) rs += mabs(fA[i + j * LA]);
-            rsum[i] = rs > 3.f ? rs : 3.f;
+            for (int j = 0; j < NX; ++j) rs += mabs(fA[i + j * ldA]);
+            m = rs > m ? rs : m;
         });
-        wone([&](int) {
-            float m = 0.f;
-            for (int i = 0; i < NX; ++i) m = rsum[i] > m ? rsum[i] : m;
-            atomic_max_u32(p.kinf + b, float_bits(m));
-        });
+        wsync();
+        merge(m);
         return;
     }
     const long long s = p.in_off[b] + t - 1;
-    const double* A = p.A + s * NX * NX;
-    const double* B = p.B + s * NX * NW;
-    const double* C = p.C + s * NY * NX;
-    const double* R = p.R + s * NR * NR;
-    const double* yt = p.yt + s * NY;
-    const double* wt = p.wt + s * NW;
-    const double* av = p.a + s * NX;
-    float* A32 = p.A32 + s * NX * NX;
-    float* B32 = p.B32 + s * NX * NW;
+    const double *A = p.A + s * NX * NX, *B = p.B + s * NX * NW, *C = p.C + s * NY * NX, *R = p.R + s * NR * NR;
+    const double *yt = p.yt + s * NY, *wt = p.wt + s * NW, *av = p.a + s * NX;
+    float *A32 = p.A32 + s * NX * NX, *B32 = p.B32 + s * NX * NW, *a32 = p.a32 + s * NX;
     // the double-float pairs of the residual (when asked for): hi = the FP32 rounding, lo = the rest
     const bool pairs = p.A_lo != nullptr;
-    float* Alo = pairs ? p.A_lo + s * NX * NX : nullptr;
-    float* Blo = pairs ? p.B_lo + s * NX * NW : nullptr;
-    float* Chi = pairs ? p.C_hi + s * NY * NX : nullptr;
-    float* Clo = pairs ? p.C_lo + s * NY * NX : nullptr;
-    float* Rhi = pairs ? p.R_hi + s * NR * NR : nullptr;
-    float* Rlo = pairs ? p.R_lo + s * NR * NR : nullptr;
-    float* a32 = p.a32 + s * NX;
     float* Qo = p.Q32 + s * NQ * NQ;
     double* lo = p.l + s * NQ;
     float* lo32 = p.l32 + s * NQ;
-    // every input block of the stage in one batched load: [C | R | A | B | y~ | w~ | a]
-    constexpr int O1 = NY * NX, O2 = O1 + NR * NR, O3 = O2 + NX * NX, O4 = O3 + NX * NW, O5 = O4 + NY + NW;
-    constexpr int TOT = O5 + NX;
-    constexpr int PER = (TOT + MHE_TEAM - 1) / MHE_TEAM;
-    wcopy<TOT, (PER + 1) / 2>(
-        [&](int i) {
-            if (i < O1) return C[i];
-            if (i < O2) return R[i - O1];
-            if (i < O3) return A[i - O2];
-            if (i < O4) return B[i - O3];
-            if (i < O4 + NY) return yt[i - O4];
-            if (i < O5) return wt[i - O4 - NY];
-            return av[i - O5];
-        },
-        [&](int i, double v) {
-            const float f = f32_rn(v);
-            if (i < O1) {
-                fC[i % NY + (i / NY) * LC] = f;
-                if (pairs) { Chi[i] = f; Clo[i] = f32_lo(v, f); }
-            } else if (i < O2) {
-                const int k = i - O1;
-                fR[k % NR + (k / NR) * LR] = f;
-                if (pairs) { Rhi[k] = f; Rlo[k] = f32_lo(v, f); }
-            } else if (i < O3) {
-                const int k = i - O2;
-                A32[k] = f;
-                fA[k % NX + (k / NX) * LA] = f;
-                if (pairs) Alo[k] = f32_lo(v, f);
-            } else if (i < O4) {
-                const int k = i - O3;
-                B32[k] = f;
-                fB[k % NX + (k / NX) * LA] = f;
-                if (pairs) Blo[k] = f32_lo(v, f);
-            } else if (i < O5) {
-                dy[i - O4] = v;   // y~ then w~ (contiguous)
-            } else {
-                a32[i - O5] = f;
-            }
-        });
-    // rows of ||K||_inf, the A and B parts: stationarity rows (a column of A or
-    // B, and -lambda_t) and dynamics rows (a row of A and of B, and -x_{t+1})
-    wfor(NQ + NX, [&](int i) {
-        float rs;
-        if (i < NX) {
-            rs = 1.f;
-            for (int j = 0; j < NX; ++j) rs += mabs(fA[j + i * LA]);
-        } else if (i < NQ) {
-            rs = 0.f;
-            for (int j = 0; j < NX; ++j) rs += mabs(fB[j + (i - NX) * LA]);
-        } else {
-            const int ii = i - NQ;
-            rs = 1.f;
-            for (int j = 0; j < NX; ++j) rs += mabs(fA[ii + j * LA]);
-            for (int j = 0; j < NW; ++j) rs += mabs(fB[ii + j * LA]);
+    // every block of the stage on its way to L2 before the first is read
+    prefetch_l2(C, 8 * NY * NX);
+    prefetch_l2(R, 8 * NR * NR);
+    prefetch_l2(A, 8 * NX * NX);
+    prefetch_l2(B, 8 * NX * NW);
+    each<NY>([&](int i) { dy[i] = yt[i]; });
+    each<NW>([&](int i) { dw[i] = wt[i]; });
+    each<NX>([&](int i) { a32[i] = f32_rn(av[i]); });
+    auto pair_out = [&](float* ho, float* lo_, int i, double v) -> float {
+        float h, l;
+        f32_pair(v, h, l);
+        if (ho) ho[i] = h;
+        if (lo_) lo_[i] = l;
+        return h;
+    };
+    float *Ch = pairs ? p.C_hi + s * NY * NX : nullptr, *Cl = pairs ? p.C_lo + s * NY * NX : nullptr;
+    float *Rh = pairs ? p.R_hi + s * NR * NR : nullptr, *Rl = pairs ? p.R_lo + s * NR * NR : nullptr;
+    float *Al = pairs ? p.A_lo + s * NX * NX : nullptr, *Bl = pairs ? p.B_lo + s * NX * NW : nullptr;
+    stream_in<NY * NX>(C, [&](int i, double v) { fC[i % NY + (i / NY) * ldC] = pair_out(Ch, Cl, i, v); });
+    stream_in<NR * NR>(R, [&](int i, double v) { fR[i / NR + (i % NR) * ldR] = pair_out(Rh, Rl, i, v); });
+    stream_in<NX * NX>(A, [&](int i, double v) { fA[i % NX + (i / NX) * ldA] = pair_out(A32, Al, i, v); });
+    stream_in<NX * NW>(B, [&](int i, double v) { fB[i % NX + (i / NX) * ldA] = pair_out(B32, Bl, i, v); });
+    wsync();
+    // rows of ||K||_inf, the A and B parts: stationarity rows (a column of A or B, and -lambda_t; the Q part
+    // follows) and dynamics rows (a row of A and of B, and -x_{t+1})
+    constexpr int RS = (NQ + MHE_TEAM - 1) / MHE_TEAM;
+    float rs[RS], m = 1.f;
+#pragma unroll
+    for (int k = 0; k < RS; ++k) {
+        const int i = lane_id() + k * MHE_TEAM;
+        rs[k] = i < NX ? 1.f : 0.f;
+        if (i < NQ) {
+#pragma unroll 8
+            for (int j = 0; j < NX; ++j) rs[k] += mabs(fA[j + i * ldA]);   // (B follows A)
         }
-        rsum[i] = rs;
+    }
+    each<NX>([&](int i) {
+        float r = 1.f;
+#pragma unroll 8
+        for (int j = 0; j < NQ; ++j) r += mabs(fA[i + j * ldA]);
+        m = r > m ? r : m;
     });
-    // FP32: V C and S C;  V(p,q) = R[NW+p + (NW+q) NR], S(k,q) = R[k + (NW+q) NR], W(k,j) = R[k + j NR]
-    wgemm<float, NY, NX, NY>([&](int, int) { return 0.f; }, [&](int i, int q) { return fR[NW + i + (NW + q) * LR]; },
-                             [&](int q, int j) { return fC[q + j * LC]; },
-                             [&](int i, int j, float v) { fVC[i + j * LC] = v; });
-    wgemm<float, NW, NX, NY>([&](int, int) { return 0.f; }, [&](int k, int q) { return fR[k + (NW + q) * LR]; },
-                             [&](int q, int j) { return fC[q + j * LC]; },
-                             [&](int k, int j, float v) { fSC[k + j * LS] = v; });
     // FP64: t = S^T w~ - V y~ (ny) and l_w = S y~ - W w~ (nw): two dot products per lane
-    wfor(NY + NW, [&](int k) {
+    each<NY + NW>([&](int k) {
         const double *m1, *v1, *m2, *v2;
         int s1, k1, s2, k2;
         if (k < NY) {
@@ -1253,42 +1249,53 @@ MHE_DEV void prep_stage(const PrepArgs& p, long long gstage, double* sm)
             lo32[NX + k - NY] = f32_rn(d);
         }
     });
-    // FP32: Q_x = C^T (V C) (one triangle, mirrored);  FP64: l_x = C^T t
-    wgemm<float, NX, NX, NY, true>([&](int, int) { return 0.f; }, [&](int i, int q) { return fC[q + i * LC]; },
-                                   [&](int q, int j) { return fVC[q + j * LC]; },
-                                   [&](int i, int j, float v) { fQx[i + j * LA] = v; fQx[j + i * LA] = v; });
-    wfor(NX, [&](int i) {
+    wsync();   // A and B are done with: Q takes their place
+    // FP32: [S; V] C (row k of R is contiguous): Q_xw = -(S C)^T and its mirror, V C
+    auto none = [](int, int) { return None(); };
+    auto put = [&](int k, int j, float v) {
+        if (k < NW) fQ[j + (NX + k) * NQ] = fQ[(NX + k) + j * NQ] = -v;
+        else fVC[k - NW + j * ldC] = v;
+    };
+    if constexpr (NX < 48) {
+        prod<float, NR, NX, NY, ldR, ldC, false, 0, MHE_TEAM>(fR + NW, fC, none,
+                                                              [&](int k, int j, float v, None) { put(k, j, v); });
+    } else {   // one term after another: the packed sums' rounding is no worse, but not the same
+        wgemm<float, NR, NX, NY>([](int, int) { return 0.f; }, [&](int k, int q) { return fR[NW + q + k * ldR]; },
+                                 [&](int q, int j) { return fC[q + j * ldC]; }, put);
+    }
+    each<NW * NW>([&](int i) { fQ[NX + i % NW + (NX + i / NW) * NQ] = fR[i / NW + (i % NW) * ldR]; });
+    wsync();
+    // Q_x = C^T (V C) (one triangle, mirrored);  FP64: l_x = C^T t
+    auto putx = [&](int i, int j, float v) { fQ[i + j * NQ] = fQ[j + i * NQ] = v; };
+    if constexpr (NX < 48) {
+        prod<float, NX, NX, NY, ldC, ldC, true, 0, MHE_TEAM>(fC, fVC, none,
+                                                             [&](int i, int j, float v, None) { putx(i, j, v); });
+    } else {
+        wgemm<float, NX, NX, NY, true>([](int, int) { return 0.f; }, [&](int i, int q) { return fC[q + i * ldC]; },
+                                       [&](int q, int j) { return fVC[q + j * ldC]; }, putx);
+    }
+    each<NX>([&](int i) {
         const double d = dot_pred<NY>(C + i * NY, 1, dt, NY, 0.0);
         lo[i] = d;
         lo32[i] = f32_rn(d);
     });
-    auto qf = [&](int i, int j) -> float {
-        if (i < NX && j < NX) return fQx[i + j * LA];
-        if (i < NX) return -fSC[(j - NX) + i * LS];
-        if (j < NX) return -fSC[(i - NX) + j * LS];
-        return fR[(i - NX) + (j - NX) * LR];
-    };
+    wsync();
     if constexpr (NQ % 4 == 0) {
-        // four consecutive rows of a column per 16-byte store
-        wfor(NQ * NQ / 4, [&](int u) {
-            const int i = 4 * (u % (NQ / 4)), j = u / (NQ / 4);
-            const float v[4] = {qf(i, j), qf(i + 1, j), qf(i + 2, j), qf(i + 3, j)};
-            st16(Qo + i + j * NQ, v);
-        });
+        each<NQ * NQ / 4>([&](int u) { st16(Qo + 4 * u, ld16g(fQ + 4 * u)); });
     } else {
-        wfor(NQ * NQ, [&](int idx) { Qo[idx] = qf(idx % NQ, idx / NQ); });
+        each<NQ * NQ>([&](int i) { Qo[i] = fQ[i]; });
     }
-    // rows of ||K||_inf: the Q part of the stationarity rows
-    wfor(NQ, [&](int i) {
-        float rs = rsum[i];
-        for (int j = 0; j < NQ; ++j) rs += mabs(qf(i, j));
-        rsum[i] = rs;
-    });
-    wone([&](int) {
-        float m = 1.f;
-        for (int i = 0; i < NQ + NX; ++i) m = rsum[i] > m ? rsum[i] : m;
-        atomic_max_u32(p.kinf + b, float_bits(m));
-    });
+#pragma unroll
+    for (int k = 0; k < RS; ++k) {
+        const int i = lane_id() + k * MHE_TEAM;
+        if (i < NQ) {
+#pragma unroll 8
+            for (int j = 0; j < NQ; ++j) rs[k] += mabs(fQ[i + j * NQ]);
+            m = rs[k] > m ? rs[k] : m;
+        }
+    }
+    wsync();
+    merge(m);
 }
 
 MHE_TEAM_NS_END
