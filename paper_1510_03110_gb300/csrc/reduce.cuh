@@ -60,7 +60,7 @@ constexpr int prod_tile(int M, int N, int LN, bool sym)
     for (int tm = 1; tm <= 6; ++tm)
         for (int tn = 1; tn <= 6; ++tn) {
             if (sym && tm != tn) continue;
-            if (tm * tn > (sizeof(T) == 8 ? 4 : 24)) continue;
+            if (tm * tn > (sizeof(T) == 8 ? 4 : 25)) continue;
             const int bm = (M + tm - 1) / tm, bn = (N + tn - 1) / tn;
             const int tasks = sym ? bm * (bm + 1) / 2 : bm * bn;
             const int rounds = (tasks + LN - 1) / LN;
