@@ -424,6 +424,33 @@ MHE_DEV float2 dot_df(const float* m, int sm, const DfVec& v)
     return make_float2(s, c);
 }
 
+// the same over a contiguous segment whose start lies a multiple of the bank count (or near it) from the
+// neighbouring lane's: lane q begins at entry q mod L and wraps, so the lanes' loads fall in different banks
+template <int L, int LO>
+MHE_DEV float2 dot_df_turn(const float* m, int q, const DfVec& v)
+{
+    Df2 a;
+    float s, c;
+    int j = q % L;
+    auto next = [&]() {
+        const int i = j;
+        j = j + 1 == L ? 0 : j + 1;
+        return i;
+    };
+#pragma unroll 4
+    for (int k = 0; k + 1 < L; k += 2) {
+        const int i0 = next(), i1 = next();
+        a.acc(pack2(m[i0], m[i1]), pack2(m[i0 + LO], m[i1 + LO]), pack2(v.p[i0], v.p[i1]),
+              pack2(v.p[v.pitch + i0], v.p[v.pitch + i1]), pack2(v.p[2 * v.pitch + i0], v.p[2 * v.pitch + i1]));
+    }
+    a.result(s, c);
+    if constexpr (L % 2 != 0) {
+        const int i = next();
+        df_acc(s, c, m[i], m[i + LO], v.p[i], v.p[v.pitch + i]);
+    }
+    return make_float2(s, c);
+}
+
 // the same over a contiguous segment, in loads of VW floats (m aligned to VW floats)
 template <int L, int LO, int VW>
 MHE_DEV float2 dot_df_col(const float* m, const DfVec& v)
@@ -615,7 +642,7 @@ MHE_DEV void resid_arrival(const ResidArgs<float>& r, int b, int N, NormMax& mx)
 // are now bound by the latency of their dependent sums (ncu: 46% issue, 51% DRAM).  Full pass, before
 // (a stage's tasks read straight from global memory, scalar instructions) and after: nx = 24, 535k
 // stages, 2.63 -> 2.06 ms; nx = 12, 1.05M stages, 2.13 -> 1.26 ms; nx = 6, 1.10M stages, 0.97 -> 0.54 ms; nx = 64,
-// 131k stages, 4.09 -> 3.96 ms.
+// 131k stages, 4.09 -> 3.17 ms (3.97 before S^T w took its columns turned: 32-way bank conflicts).
 template <int NX, int NW, int NY, class IT>
 MHE_DEV void resid_df_run(const ResidArgs<float>& r, IT& it, unsigned char* smem)
 {
@@ -690,8 +717,14 @@ MHE_DEV void resid_df_run(const ResidArgs<float>& r, IT& it, unsigned char* smem
         });
         wsync();
         // segments of C x, then W w and S^T w (the first nw entries of column nw + k of R)
+        // (at nx >= 48 a column of R is a multiple of the banks long: S^T w goes apart, turned)
+        constexpr bool turn = NR % 32 == 0;
+        if constexpr (turn)
+            rounds(0, NY, [&](int k) {
+                pr[S::sw + k] = dot_df_turn<NW, S::crl>(cr + S::oR + (NW + k) * NR, k, zv(S::sw0));
+            });
         if constexpr (LP == NW) {
-            rounds(0, NY * SP + NW + NY, [&](int k) {
+            rounds(0, NY * SP + NW + (turn ? 0 : NY), [&](int k) {
                 const float* m;
                 int sm, j0, o;
                 if (k < NY * SP) {
@@ -719,7 +752,7 @@ MHE_DEV void resid_df_run(const ResidArgs<float>& r, IT& it, unsigned char* smem
                 const int j0 = (k / NY) * LP;
                 pr[S::cx + k] = dot_df<LP, S::crl>(cr + k % NY + j0 * ldC, ldC, zv(j0));
             });
-            rounds(0, NR, [&](int k) {
+            rounds(0, turn ? NW : NR, [&](int k) {
                 const bool w = k < NW;
                 pr[w ? S::ww + k : S::sw + k - NW] =
                     dot_df<NW, S::crl>(cr + S::oR + (w ? k : k * NR), w ? NR : 1, zv(S::sw0));

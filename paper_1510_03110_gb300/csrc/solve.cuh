@@ -257,11 +257,12 @@ inline int device_sms()
 
 // CTAs per instance of a fused solve for a batch whose longest horizon is max_N, or 0 for a launch
 // per level pass.  The clusters together about fill the chip once, and a team has at least about
-// one stage of the residual.  A team that would walk more than 16 stages per residual, or a batch of more
-// instances than SMs, keeps the chip busy with a launch per pass, which spreads the chunks of all
-// instances evenly.  (Measured: 256 instances of nx = 12, N <= 512: 2.0 ms per pass, 2.4 ms fused; 79 of
-// N <= 160: 0.99 and 0.55 ms; one of nx = 24, N = 1000 on 16 CTAs, 8 stages a team: 1.72 and 1.49 ms; one
-// of nx = 20, N = 16384 in FP64, 256 stages a team: 10.5 and 13.7 ms.)
+// one stage of the residual.  A team that would walk more than 16 stages per residual (six for nx > 12, whose
+// stages are longer), or a batch of more instances than SMs, keeps the chip busy with a launch per pass, which
+// spreads the chunks of all instances over all SMs.  Measured, launches per pass and fused: 79 instances of nx =
+// 12, N <= 160: 0.99 and 0.55 ms; one of nx = 12, N = 200: 0.36 and 0.29 ms; one of nx = 12, N = 1621 in FP64, 13 stages a
+// team: 0.85 and 0.82 ms; one of nx = 24, N = 1000, 8 stages a team: 0.85 and 0.96 ms; 256 of nx = 12, N <= 512: 1.32
+// and 2.17 ms; one of nx = 20, N = 16384 in FP64, 256 stages a team: 3.6 and 7 ms.
 template <int NX, int NW, int NY>
 int solve_cluster(int fp64, int batch, int max_N)
 {
@@ -271,7 +272,7 @@ int solve_cluster(int fp64, int batch, int max_N)
     if (batch > room || most < 1) return 0;
     int c = 1;
     while (c * 2 <= most && batch * c * 2 <= room && (long long)c * 2 * teams * 10 <= (long long)max_N * 13) c *= 2;
-    return max_N <= 16 * c * teams ? c : 0;
+    return max_N <= (NX <= 12 ? 16 : 6) * c * teams ? c : 0;
 }
 
 MHE_TEAM_NS_END
