@@ -348,7 +348,8 @@ int mhe_server_stats(mhe_server* s, long long* out, int cap);
 int mhe_server_destroy(mhe_server* s);
 
 /* Profiling aid: enable = 1 records a pair of CUDA events around every level
- * pass (reduce, right-hand side, down, residual) on the context's stream;
+ * pass (reduce, right-hand side, down, residual) on the context's stream, each
+ * pass a launch of its own (a solve that runs as one launch is split);
  * enable = 0 stops recording.  No counterpart in the paper, whose Matlab
  * experiment timed each tree level the same way (Section VI). */
 int mhe_timing_enable(mhe_ctx* ctx, int enable);

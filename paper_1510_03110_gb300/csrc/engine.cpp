@@ -490,6 +490,7 @@ void Engine::reduce_level(int k, const T* A_, const T* B_, const T* Q_, const T*
     launches += g.nchunks > 0;
     auto r32 = ops->reduce32;
     if (prec == MHE_TF32_IR && ops->reduce32tc) r32 = ops->reduce32tc;
+    if (prec == MHE_TF32_IR && ops->reduce32tc1 && lv.size() == 1) r32 = ops->reduce32tc1;   // every chunk a whole instance
     if (prec == MHE_BF16_IR && ops->reduce32bf) r32 = ops->reduce32bf;
     const bool tc = r32 != ops->reduce32;   // the tensor-core reductions have their own team
     if (sizeof(T) == 8 ? (ops->reduce64w && g.nchunks <= ops->wide64)

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "engine.h"
+#include "reduce_tc.cuh"
 #include "resid.cuh"
 #include "solve.cuh"
 #include "tree.cuh"
@@ -98,14 +99,9 @@ constexpr int level_threads()
     return vector_op<OP>() ? 128 : (OP == OP_REDUCE && small_shape<NX>() ? level_warps<T, NX, NW, UPPER, OP>() * MHE_TEAM : 256);
 }
 
-// CTAs of 256 threads per SM the register allocation is sized for: the small
-// shapes' workspaces are small, so their occupancy is set by registers (64 or
-// 80 per thread keep 32 or 24 warps per SM); the n = 24 reduction keeps its
-// 255 registers (shared memory allows one CTA anyway), its right-hand-side pass
-// 128 and its down pass 85 (measured: the down pass gains from a third CTA,
-// the right-hand-side pass, whose loads are unrolled wider, loses);
-// the n = 64 passes (one four-warp team per subproblem, a few hundred teams)
-// all take 255.
+// CTAs per SM the register allocation is sized for.  The literal Algorithm 6 pass (nx <= 32, 256 threads, the
+// general workspace): 64 or 80 registers a thread keep 32 or 24 warps per SM of the small shapes, nx = 20 and
+// 24 keep 255 (shared memory allows one CTA anyway); the nx = 64 passes of four-warp teams take 255.
 template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int level_min_blocks()
 {
@@ -122,11 +118,7 @@ constexpr int level_min_blocks()
         constexpr int regs = 65536 / (w * MHE_TEAM * 96);
         return fit < regs ? (fit < 1 ? 1 : fit) : (regs < 1 ? 1 : regs);
     }
-    return NX >= 48 ? 1   // four-warp teams, a few per SM: every pass may take 255 registers
-                    : (sizeof(T) == 4
-                           ? (NX <= 8 ? 4
-                                      : (NX <= 12 ? 3 : ((OP == OP_REDUCE || OP >= OP_REDUCE_TC) ? 1 : (OP == OP_DOWN ? 3 : 2))))
-                           : (NX <= 12 ? 2 : ((OP == OP_REDUCE || OP == OP_DOWN_LIT) ? 1 : 2)));
+    return NX > 12 ? 1 : (sizeof(T) == 8 ? 2 : (NX <= 8 ? 4 : 3));
 }
 
 // shapes whose stage products run on the tensor cores: a team of four warps,
@@ -191,18 +183,13 @@ __global__ void __launch_bounds__(level_threads<T, NX, NW, UPPER, OP>(), level_m
         __syncthreads();
         tc::fence_after();
         if (threadIdx.x < 32) tc::tmem_dealloc(tcs.tbase, 512);
-    } else if (!chunk_in_bounds(a, ci)) {
-        return;
-    } else if constexpr (OP == OP_REDUCE && small_shape<NX>()) {
-        reduce_chunk_small<T, NX, NW, UPPER != 0>(a, ci, sm);
-    } else if (OP == OP_REDUCE) {
-        reduce_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
-    } else if (OP == OP_RHS) {
-        rhs_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
-    } else if (OP == OP_DOWN_LIT) {
-        down_chunk_literal<T, NX, NW, UPPER != 0>(a, ci, sm);
     } else {
-        down_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
+        if (!chunk_in_bounds(a, ci)) return;
+        if constexpr (OP == OP_REDUCE && small_shape<NX>()) reduce_chunk_small<T, NX, NW, UPPER != 0>(a, ci, sm);
+        else if constexpr (OP == OP_REDUCE) reduce_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
+        else if constexpr (OP == OP_RHS) rhs_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
+        else if constexpr (OP == OP_DOWN_LIT) down_chunk_literal<T, NX, NW, UPPER != 0>(a, ci, sm);
+        else down_chunk<T, NX, NW, UPPER != 0>(a, ci, sm);
     }
 }
 
@@ -236,6 +223,49 @@ void launch_level(const LevelArgs<T>& a, int upper, void* stream)
     else launch_level_v<T, NX, NW, 0, OP>(a, stream);
 }
 
+// Whole instances (plans of one level), TF32 products: two CTAs of one team per SM.  Measured (nx = 64, 256
+// instances of 512 stages): 18.04 -> 9.9 ms, a step 45.7 -> 37.5 ms.  Plans of several levels keep the general
+// workspace: their other chunks' stages form V.
+constexpr int kTcLastCols = 256;   // TMEM columns of a team: half of an SM's
+
+template <int NX, int NW>
+__global__ void __launch_bounds__(MHE_TEAM, 2) k_reduce_last(LevelArgs<float> a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (a.any_active && *a.any_active == 0) return;
+    float* sm = reinterpret_cast<float*>(smem_raw);
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + TcWs<NX, NW>::count);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(mbar + 1);
+    static_assert(2 * (NX + NW) <= kTcLastCols && TcWs<NX, NW>::count % 4 == 0, "accumulators, alignment");
+    if (threadIdx.x < 32) tc::tmem_alloc(slot, kTcLastCols);
+    if (threadIdx.x == 0) tc::mbar_init(mbar, 1);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    TcState tcs{*slot, mbar, nullptr, 0u, 1};
+    if (chunk_in_bounds(a, blockIdx.x)) reduce_last_tc<NX, NW>(a, blockIdx.x, sm, tcs);
+    // a wait that ran out: give the MMAs of that phase another bounded wait before freeing TMEM
+    if (!tcs.ok) tc::mbar_wait(mbar, tcs.phase, tc::kWaitLimit);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (threadIdx.x < 32) tc::tmem_dealloc(tcs.tbase, kTcLastCols);
+}
+
+template <int NX, int NW>
+void launch_reduce_last(const LevelArgs<float>& a, int, void* stream)
+{
+    if (a.nchunks <= 0) return;
+    constexpr size_t smem = (size_t)TcWs<NX, NW>::count * sizeof(float) + 16;
+    static_assert(2 * (smem + 1024) <= 228 * 1024, "two CTAs per SM");
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(k_reduce_last<NX, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        attr = true;
+    }
+    k_reduce_last<NX, NW><<<a.nchunks, MHE_TEAM, smem, (cudaStream_t)stream>>>(a);
+}
+
 // The residual waits on its FP64 loads from HBM; five CTAs of 256 threads per SM
 // (48 registers a thread, a few spilled) hide that latency better than four.
 template <int NX, int NW, typename TR, int NY>
@@ -249,8 +279,8 @@ __global__ void __launch_bounds__(256, kResidBlocks) k_resid(ResidArgs<TR> r)
     resid_stage<NX, NW, TR, NY>(r, g, sm[team]);
 }
 
-// The double-float residual (MHE form, FP32 correction solves): one resident grid of CTAs of up to
-// 128 threads (their workspaces fill an SM's shared memory), whose teams walk the stages.
+// The double-float residual (MHE form, FP32 correction solves): one resident grid of small CTAs
+// (their workspaces fill an SM's shared memory), whose teams walk the stages.
 template <int NX, int NW, int NY>
 constexpr int resid_df_teams()
 {
@@ -423,6 +453,8 @@ ShapeEntry make_shape()
         e.ops.reduce32tc = nullptr;
         e.ops.reduce32bf = nullptr;
     }
+    if constexpr (tc_shape<NX, NW>() && tc_last_shape<NX, NW>()) e.ops.reduce32tc1 = &launch_reduce_last<NX, NW>;
+    else e.ops.reduce32tc1 = nullptr;
     e.ops.rhs32 = &launch_level<float, NX, NW, OP_RHS>;
     e.ops.down32 = &launch_level<float, NX, NW, OP_DOWN>;
     // the literal Algorithm 6 down pass, for the shapes whose reduction workspace fits an SM

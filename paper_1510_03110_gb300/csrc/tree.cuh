@@ -1,9 +1,10 @@
-// tree.cuh -- warp-per-subproblem bodies of the parallel Riccati tree.
+// tree.cuh -- the general stage of the parallel Riccati tree: shapes of more than 32 states,
+// the tensor-core stage products, and Algorithm 6 as printed.
 //
-// One warp owns one subproblem (chunk) of one level and walks its stages
-// serially; inside a stage the lanes share the small dense products.  All
-// per-chunk state (P, Psi, V, v, Q^_w) and the stage's A_t, B_t live in shared
-// memory; Q_t and l_t are read from global memory inside the products.
+// One team owns one subproblem (chunk) of one level and walks its stages serially;
+// inside a stage the lanes share the small dense products.  All per-chunk state
+// (P, Psi, V, v, Q^_w) and the stage's A_t, B_t live in the workspace; Q_t and l_t
+// are read from global memory inside the products.
 //
 //   reduce_chunk  Algorithm 4 (matrix part always; vector part when a
 //                 right-hand side is given).  Non-last chunks emit the master
@@ -12,18 +13,11 @@
 //                 R^T R = Q^_w = B^); the last chunk of a level is factored with its
 //                 known terminal (Algorithms 1-2) and emits the next level's
 //                 terminal cost (Q^_x,p = P_0, l^_x,p = -Psi_0); the top chunk
-//                 emits nothing.
-//   rhs_chunk     the vector part of Algorithm 4 alone with stored factors
-//                 (k, Psi, and a^ by simulating the closed loop
-//                 x_{t+1} = (A + B K_0) x_t + a + B k_0 from x = 0, which is
-//                 Eq. a).
-//   down_chunk    the solution of one subproblem from its parent's x^_i, w^_i
-//                 (= R^{-1} w^'_i) and lambda^_{i+1}: w_t = k_0 + K_0 x_t - L_{t+1} w^_i
-//                 (Eq. control_signal_def with the T-form reduced input),
-//                 x_{t+1} = A x + B w + a, then the costate sweep
-//                 lambda_t = Q_x x_t + Q_xw w_t + l_x + A^T lambda_{t+1}.
-//   resid_stage   KKT residual rows of one stage (FP64).
-//   assemble_stage  MHE weights -> UFTOC Q_t, l_t, c_t (Section II).
+//                 emits nothing.  reduce.cuh has it for at most 32 states.
+//   down_chunk_literal  Algorithm 6 as printed (every subproblem solved again).
+//
+// vec.cuh has the vector passes over stored factors (rhs_chunk, down_chunk),
+// resid.cuh the stage assembly and the KKT residual.
 #pragma once
 #include <stdint.h>
 #include <type_traits>
@@ -64,34 +58,6 @@ struct Ws {
         sc = p;
     }
 };
-
-// init + sum_{p<K} fa(p) fb(p) with four independent accumulators (the
-// products of one stage are short dot products; four chains hide the FMA latency)
-template <int K, typename T, class FA, class FB>
-MHE_DEV T dot4(T init, FA&& fa, FB&& fb)
-{
-    T a0 = init, a1 = 0, a2 = 0, a3 = 0;
-#pragma unroll
-    for (int p = 0; p + 3 < K; p += 4) {
-        a0 += fa(p) * fb(p);
-        a1 += fa(p + 1) * fb(p + 1);
-        a2 += fa(p + 2) * fb(p + 2);
-        a3 += fa(p + 3) * fb(p + 3);
-    }
-#pragma unroll
-    for (int p = K & ~3; p < K; ++p) a0 += fa(p) * fb(p);
-    return (a0 + a1) + (a2 + a3);
-}
-
-// upper-triangle index -> (i <= j)
-MHE_DEV void tri_ij(int idx, int& i, int& j)
-{
-    int jj = (int)((msqrt(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
-    while ((jj + 1) * (jj + 2) / 2 <= idx) ++jj;
-    while (jj * (jj + 1) / 2 > idx) --jj;
-    j = jj;
-    i = idx - jj * (jj + 1) / 2;
-}
 
 // A -> s.A, B -> s.B, a -> s.e.  FP32 blocks stored in memory (leaf and master
 // stages) move in 16-byte pieces when n is a multiple of four: a column of A or
@@ -170,7 +136,8 @@ MHE_DEV bool chol_inplace(Ws<T, NX>& s, T* Gm, double piv_rel)
     constexpr int ld = Ws<T, NX>::ld;
     if constexpr (M <= 32) {
         // rows in the registers of one warp, columns passed by shuffles
-        team_chol<T, M, INV>(Gm, ld, piv_rel, s.sc + 1);
+        static_assert(INV, "reciprocal pivots");
+        team_chol<T, M>(Gm, ld, piv_rel, s.sc + 1);
         return s.sc[1] != 0;
     }
     wone([&](int) { s.sc[1] = 0; });
@@ -283,7 +250,6 @@ MHE_DEV void upper_solve(const Ws<T, NX>& s, FR&& rhs, FG&& get, FP&& put)
     });
 }
 
-
 // Y = L^{-1} R and (when upper) X = L^{-T} Y for pivots blocks of at most 16
 // rows: one right-hand-side column per lane, held in registers through both
 // substitutions (the factor read by broadcast from shared memory), so the two
@@ -323,27 +289,13 @@ template <typename T, int NX, int M>
 MHE_DEV void store_inverse(Ws<T, NX>& s, T* dst)
 {
     constexpr int ld = Ws<T, NX>::ld;
-    if constexpr (M <= 24) {
-        wfor(M, [&](int c) {   // column c of L^{-1} in registers
-            T y[M];
-#pragma unroll
-            for (int i = 0; i < M; ++i) {
-                T acc = i == c ? (T)1 : (T)0;
-#pragma unroll
-                for (int p = 0; p < i; ++p) acc -= s.G[i + p * ld] * y[p];
-                y[i] = acc * s.G[i + i * ld];
-                dst[c + i * M] = y[i];
-            }
-        });
-    } else {
-        lower_solve<T, NX, M, M>(s, [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); },
-                                 [&](int i, int c) -> T { return s.H[i + c * ld]; },
-                                 [&](int i, int c, T v) { s.H[i + c * ld] = v; });
-        wfor(M * M, [&](int r) {
-            const int c = r % M, i = r / M;
-            dst[r] = i >= c ? s.H[i + c * ld] : (T)0;
-        });
-    }
+    lower_solve<T, NX, M, M>(s, [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); },
+                             [&](int i, int c) -> T { return s.H[i + c * ld]; },
+                             [&](int i, int c, T v) { s.H[i + c * ld] = v; });
+    wfor(M * M, [&](int r) {
+        const int c = r % M, i = r / M;
+        dst[r] = i >= c ? s.H[i + c * ld] : (T)0;
+    });
 }
 
 // ---- the stage products on the tensor cores (tcgen05, kind::tf32) -------------
@@ -835,12 +787,8 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
         auto putZ = [&](int i, int c, T v) { s.PB[i + c * ld] = v; };
         auto getL = [&](int i, int c) -> T { return s.Tt[i + c * ld]; };
         auto putL = [&](int i, int c, T v) { s.Tt[i + c * ld] = v; };
-        if constexpr (MT <= 16) {
-            col_solves<T, NX, MT, NX>(s, Lout != nullptr, rhsZ, putZ, putL);
-        } else {
-            lower_solve<T, NX, MT, NX>(s, rhsZ, getZ, putZ);
-            if (Lout) upper_solve<T, NX, MT, NX>(s, getZ, getL, putL);
-        }
+        lower_solve<T, NX, MT, NX>(s, rhsZ, getZ, putZ);
+        if (Lout) upper_solve<T, NX, MT, NX>(s, getZ, getL, putL);
         if (Lout) store_block<T, MT, NX, ld>(Lout, s.Tt, (T)-1, 0, [](int) {});
     }
     // V_new = A^T V + K^T BV -> Tt;  Q^_w += Z^T Z (symmetric)

@@ -192,14 +192,6 @@ MHE_DEV void atomic_max_u64(unsigned long long* addr, unsigned long long v) { at
 MHE_DEV void atomic_max_u32(unsigned int* addr, unsigned int v) { atomicMax(addr, v); }
 MHE_DEV unsigned int float_bits(float v) { return __float_as_uint(v); }
 
-// max of non-negative doubles through their bit patterns (ordered like the values)
-MHE_DEV void atomic_max_nonneg(double* addr, double v)
-{
-    if (!(v >= 0.0)) v = __longlong_as_double(0x7ff8000000000000LL);   // NaN: keep it visible
-    atomicMax(reinterpret_cast<unsigned long long*>(addr),
-              static_cast<unsigned long long>(__double_as_longlong(v)));
-}
-
 // In-place Cholesky G = L L^T of the M x M matrix at Gm (lower triangle read
 // and written, leading dimension ld), M <= 32: one row per lane of the team's
 // first warp (or of the team, when it is narrower), the row held in registers,
@@ -209,10 +201,9 @@ MHE_DEV void atomic_max_nonneg(double* addr, double v)
 // subtracts L_ij L_cj from its entries c = j+1..i.  A pivot that is not above
 // piv_rel * G_jj (column j's own diagonal before elimination: a test that a
 // diagonal scaling of G leaves unchanged) is replaced by 1 and reported:
-// *flag = 1 (else 0), written by lane 0 before the closing team barrier.  INV stores 1 / L_jj on
-// the diagonal and multiplies by it, 1 / L_jj from the reciprocal square root
-// of the pivot; otherwise L_jj is stored and the column divided.
-template <typename T, int M, bool INV>
+// *flag = 1 (else 0), written by lane 0 before the closing team barrier.  The diagonal
+// holds 1 / L_jj, from the reciprocal square root of the pivot.
+template <typename T, int M>
 MHE_DEV void team_chol(T* Gm, int ld, double piv_rel, T* flag)
 {
     constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32;
@@ -234,16 +225,9 @@ MHE_DEV void team_chol(T* Gm, int ld, double piv_rel, T* flag)
                 bad = 1;
                 d = (T)1;
             }
-            T lij;
-            if constexpr (INV) {
-                const T inv = mrsqrt(d);   // 1 / L_jj in one step (the refinement absorbs its rounding)
-                lij = g[j] * inv;
-                if (i == j) g[j] = inv;
-            } else {
-                const T l = msqrt(d);
-                lij = g[j] / l;
-                if (i == j) g[j] = l;
-            }
+            const T inv = mrsqrt(d);   // 1 / L_jj in one step (the refinement absorbs its rounding)
+            const T lij = g[j] * inv;
+            if (i == j) g[j] = inv;
             const T lv = i > j ? lij : (T)0;
             if (i > j) g[j] = lij;
 #pragma unroll

@@ -101,3 +101,45 @@ def test_preparation_of_zeros_and_extreme_entries():
     assert np.all(info["status"] == 0)
     for sol, p in zip(split(*out, d["N"], n, m), insts):
         assert rel_err(sol, oracle.riccati(oracle.mhe_to_uftoc(p))) <= 1e-8
+
+
+@pytest.mark.parametrize("first_only", [True, False])
+def test_whole_instances_on_the_tensor_cores(first_only):
+    """nx = 64, TF32 products, plans of one level: more instances than two teams an SM, horizons from the arrival
+    stage alone up; factors kept for another right-hand side.  The first solve's error against FP32's:
+    the split products are as accurate as an FP32 chain (2.0e-7 against 1.8e-7 of sum |ab|), everything
+    after them is the same arithmetic in another order; a factor 8 is left for the order."""
+    n, m = 64, 32
+    Ns = [1 + i % 4 for i in range(320)] + [33]
+    insts = [synth.mhe_instance(4900 + i % 24, n, m, m, N) for i, N in enumerate(Ns)]
+    d = device_inputs(insts)
+    err = {}
+    for prec in (mhe.MHE_TF32_IR, mhe.MHE_FP32_IR):
+        out, info, _ = _run(d, "solve", prec, False, top_len=1000, refine_tol=1e-13,
+                            max_refine=0 if first_only else 20)
+        sols = split(*out, Ns, n, m)
+        for b in list(range(4)) + [303, 304, 319, 320]:
+            e = rel_err(sols[b], oracle.riccati(oracle.mhe_to_uftoc(insts[b])))
+            err[prec, b] = e
+            if not first_only:
+                assert info["status"][b] == 0 and e <= 1e-8, (prec, b, e, info[b])
+    if first_only:
+        most = {p: max(e for (q, _), e in err.items() if q == p) for p in (mhe.MHE_TF32_IR, mhe.MHE_FP32_IR)}
+        assert most[mhe.MHE_TF32_IR] <= 8 * most[mhe.MHE_FP32_IR], most
+
+
+@pytest.mark.parametrize("where", [0, 1, 4])
+def test_failed_pivot_of_a_whole_instance_on_the_tensor_cores(where):
+    """The failed stage (the arrival stage, the first and the last measured one) is reported for its instance only."""
+    n, m, N = 64, 32, 5
+    insts = [synth.mhe_instance(5000 + i, n, m, m, N) for i in range(3)]
+    d = device_inputs(insts)
+    if where == 0:
+        d["P0inv"].view(3, n * n)[1].mul_(-1e6)
+    else:
+        import torch
+        q = d["Q"].view(3, N - 1, n + m, n + m)[1, where - 1]
+        q[n:, n:] = -1e6 * torch.eye(m, dtype=torch.float64, device="cuda")
+    _, info, _ = _run(d, "solve", mhe.MHE_TF32_IR, False, top_len=1000, refine_tol=1e-12, max_refine=4)
+    assert info["status"][1] == -3 and info["stage"][1] == where and info["chunk"][1] == 1, info[1]
+    assert info["status"][0] == 0 and info["status"][2] == 0
