@@ -33,11 +33,11 @@ constexpr bool small_shape() { return NX <= 32; }
 template <typename T, int NX, int NW, int UPPER, int OP>
 constexpr int op_count()
 {
-    if (OP == OP_REDUCE && small_shape<NX>()) return RedWs<T, NX, NW, UPPER != 0>::count;
+    if (OP == OP_REDUCE && small_shape<NX>()) return team_stride<T>(RedWs<T, NX, NW, UPPER != 0>::count);
     return (OP == OP_REDUCE || OP == OP_DOWN_LIT)
                ? Ws<T, NX>::count
-               : (OP == OP_RHS ? VecWs<T, NX, NW, UPPER != 0>::rhs_count
-                               : (OP == OP_DOWN ? VecWs<T, NX, NW, UPPER != 0>::down_count
+               : (OP == OP_RHS ? team_stride<T>(VecWs<T, NX, NW, UPPER != 0>::rhs_count)
+                               : (OP == OP_DOWN ? team_stride<T>(VecWs<T, NX, NW, UPPER != 0>::down_count)
                                                 : Ws<T, NX>::count + kTcExtra));   // both tensor-core reductions
 }
 
@@ -279,19 +279,18 @@ __global__ void __launch_bounds__(256, kResidBlocks) k_resid(ResidArgs<TR> r)
     resid_stage<NX, NW, TR, NY>(r, g, sm[team]);
 }
 
-// The double-float residual (MHE form, FP32 correction solves): one resident grid of small CTAs
-// (their workspaces fill an SM's shared memory), whose teams walk the stages.
+// The double-float residual (MHE form, FP32 correction solves): one resident grid, whose teams walk the
+// stages, in CTAs that leave the least of an SM's shared memory unused (at most 64 threads a CTA before: nx = 24,
+// 535k stages, 2.05 -> 1.94 ms; nx = 12, 1.05M stages, 1.27 -> 1.22 ms).
 template <int NX, int NW, int NY>
-constexpr int resid_df_teams()
-{
-    constexpr int fit = 113 * 1024 / DfWs<NX, NW, NY>::bytes, most = MHE_TEAM >= 64 ? 1 : 64 / MHE_TEAM;
-    return fit < 1 ? 1 : (fit < most ? fit : most);
-}
+constexpr int resid_df_teams() { return best_teams(DfWs<NX, NW, NY>::bytes); }
 template <int NX, int NW, int NY>
 constexpr int resid_df_blocks()
 {
-    constexpr int fit = 228 * 1024 / (resid_df_teams<NX, NW, NY>() * DfWs<NX, NW, NY>::bytes + 1024);
-    return fit > 16 ? 16 : (fit < 1 ? 1 : fit);
+    // what shared memory holds, with at least 64 registers a thread
+    constexpr int w = resid_df_teams<NX, NW, NY>();
+    constexpr int fit = ctas_per_sm(w, DfWs<NX, NW, NY>::bytes), regs = 65536 / (w * MHE_TEAM * 64);
+    return fit < regs ? (fit < 1 ? 1 : fit) : (regs < 1 ? 1 : regs);
 }
 
 template <int NX, int NW, int NY>
@@ -335,11 +334,8 @@ void launch_resid(const ResidArgs<TR>& r, void* stream)
 template <int NX, int NW, int NY>
 constexpr int prep_warps()
 {
-    return (40 * 1024) / (int)(PrepSmem<NX, NW, NY>::count * 8) >= kMaxTeams
-               ? kMaxTeams
-               : ((40 * 1024) / (int)(PrepSmem<NX, NW, NY>::count * 8) < 1
-                      ? 1
-                      : (40 * 1024) / (int)(PrepSmem<NX, NW, NY>::count * 8));
+    constexpr int fit = 40 * 1024 / (PrepSmem<NX, NW, NY>::count * 8);
+    return fit >= kMaxTeams ? kMaxTeams : (fit < 1 ? 1 : fit);
 }
 
 template <int NX, int NW, int NY>

@@ -196,7 +196,7 @@ struct RedWs {
     static constexpr int lm0 = pick_ld(NX, vec_of<T>(NX));
     static constexpr int a_end = S::oS + round_to(lm0 * (NX + 1), V) + 2 * round_to(lm0 * NX, V);
     static constexpr int vec = UPPER ? S::end : max_int(S::end, a_end);
-    static constexpr int count = vec + 6 * nv + round_to(8, V);   // Psi, v, t, va, w1, w2; flags
+    static constexpr int count = vec + 5 * nv + round_to(8, V);   // Psi, v, t, va, thr; flags
 };
 
 // G = L L^T for the M x M block at G (by columns, leading dimension LD, both triangles or the lower one given).
@@ -480,7 +480,7 @@ MHE_DEV void load_stage(T* W, const StageRef<T>& st)
 // Workspace pointers of a chunk's sweep
 template <typename T>
 struct RedPtr {
-    T *P, *Qw, *V, *X, *W, *Y, *Z, *G, *R, *Psi, *v, *t, *va, *thr, *w2, *flag;
+    T *P, *Qw, *V, *X, *W, *Y, *Z, *G, *R, *Psi, *v, *t, *va, *thr, *flag;
 };
 
 // One backward stage (see above).  want_v: V, v and Q^_w are carried and L_t stored.  after3() runs once A, B
@@ -647,7 +647,7 @@ MHE_DEV void reduce_chunk_small(const LevelArgs<T>& a, int ci, T* smem)
     s.W = smem + S::oW; s.Y = smem + S::oY; s.Z = smem + S::oZ; s.G = smem + S::oG; s.R = smem + S::oR;
     T* vec = smem + WS::vec;
     s.Psi = vec; s.v = vec + WS::nv; s.t = vec + 2 * WS::nv; s.va = vec + 3 * WS::nv; s.thr = vec + 4 * WS::nv;
-    s.w2 = vec + 5 * WS::nv; s.flag = vec + 6 * WS::nv;
+    s.flag = vec + 5 * WS::nv;
     const T* QN = UPPER ? a.QNk + (long long)b * NX * NX : nullptr;   // level 0: Q_{x,N} = 0
     const T* lN = UPPER ? (a.lNk ? a.lNk + (long long)b * NX : nullptr)
                         : (a.lN ? a.lN + (long long)b * NX : nullptr);

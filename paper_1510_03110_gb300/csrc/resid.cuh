@@ -1135,13 +1135,15 @@ struct PrepSmem {
     static_assert(NW % vec_of<float>(NY) == 0, "the S and V parts of a row of R start on a whole vector");
 };
 
-// f(i, src[i]) for i < COUNT, lanes round-robin, the next eight loads of a lane in flight while it works on eight.
-// The rounds are not unrolled: a preparation stage unrolled in full outgrows the instruction cache (at nx = 64
-// ten of thirteen warp cycles per instruction went into waiting for instructions).
+// f(i, src[i]) for i < COUNT, lanes round-robin, the next loads of a lane (MOST of them) in flight while it works
+// on as many.  The rounds are not unrolled: a preparation stage unrolled in full outgrows the instruction cache
+// (at nx = 64 ten of thirteen warp cycles per instruction went into waiting for instructions).  MOST: nx = 24,
+// 535k stages, 4.09 ms with 4, 3.51 with 6, 4.01 with 12; nx = 64, 131k stages, 11.42 with 2, 9.82 with 4, 10.94 with
+// 6, 11.86 with 12.
 template <int COUNT, class F>
 MHE_DEV void stream_in(const double* src, F&& f)
 {
-    constexpr int PER = (COUNT + MHE_TEAM - 1) / MHE_TEAM, CH = PER < 6 ? PER : 6, NB = (PER + CH - 1) / CH;
+    constexpr int PER = (COUNT + MHE_TEAM - 1) / MHE_TEAM, MOST = MHE_TEAM >= 128 ? 4 : 6, CH = PER < MOST ? PER : MOST, NB = (PER + CH - 1) / CH;
     double cur[CH], nxt[CH];
     auto load = [&](double (&v)[CH], int k0) {
 #pragma unroll

@@ -33,7 +33,8 @@ constexpr int solve_words()
     constexpr int v = max_int(max_int(V0::rhs_count, V0::down_count), max_int(V1::rhs_count, V1::down_count));
     constexpr int r = (v * (int)sizeof(T) + 7) / 8;
     constexpr int q = NY > 0 ? DfWs<NX, NW, NY == 0 ? 1 : NY>::bytes / 8 : ResidSmem<NX, NW, 0>::count;
-    return ((r > q ? r : q) + 1) / 2 * 2;
+    constexpr int n = ((r > q ? r : q) + 1) / 2 * 2;
+    return team_stride<T>(n * (8 / (int)sizeof(T))) * (int)sizeof(T) / 8;
 }
 
 // teams per CTA: 256 threads, fewer (a power of two) where their workspaces do not fit

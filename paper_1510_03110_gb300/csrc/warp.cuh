@@ -41,6 +41,15 @@ MHE_DEV int lane_id() { return threadIdx.x & (MHE_TEAM - 1); }
 // index of the team within its CTA
 MHE_DEV int team_id() { return threadIdx.x / MHE_TEAM; }
 
+// A workspace of n entries of T, lengthened so that the teams of one warp start in distinct bank groups: an odd
+// multiple of the team's width.  (At nx = 6 a multiple of 16 words, two of a warp's four teams in the same
+// banks, took the leaf reduction from 0.55 to 0.66 ms.)
+template <typename T>
+constexpr int team_stride(int n)
+{
+    return MHE_TEAM * (int)sizeof(T) >= 128 ? n : (((n + MHE_TEAM - 1) / MHE_TEAM) | 1) * MHE_TEAM;
+}
+
 // Barrier of the team's lanes: __syncwarp over the team's lanes within a warp,
 // a named barrier (team_id + 1) when a team is several warps.
 MHE_DEV void wsync()
