@@ -1,9 +1,8 @@
 // kernels.cuh -- __global__ wrappers and launchers of the level passes.
 //
-// Launch shape: one team (MHE_TEAM lanes) per chunk, W teams per CTA where W is
-// the number of per-team shared-memory workspaces that fit in kLevelSmem (at
-// most 256 threads per CTA); the tensor-core reductions take one four-warp team
-// per CTA.
+// Launch shape: one team (MHE_TEAM lanes) per chunk, W teams per CTA (at most 256
+// threads) by the shared memory their workspaces take; the tensor-core reductions
+// take one four-warp team per CTA.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -224,7 +223,7 @@ void launch_level(const LevelArgs<T>& a, int upper, void* stream)
 }
 
 // Whole instances (plans of one level), TF32 products: two CTAs of one team per SM.  Measured (nx = 64, 256
-// instances of 512 stages): 18.04 -> 9.9 ms, a step 45.7 -> 37.5 ms.  Plans of several levels keep the general
+// instances of 512 stages): 18.04 -> 9.9 ms, the estimate 45.7 -> 37.5 ms.  Plans of several levels keep the general
 // workspace: their other chunks' stages form V.
 constexpr int kTcLastCols = 256;   // TMEM columns of a team: half of an SM's
 
@@ -281,7 +280,7 @@ __global__ void __launch_bounds__(256, kResidBlocks) k_resid(ResidArgs<TR> r)
 
 // The double-float residual (MHE form, FP32 correction solves): one resident grid, whose teams walk the
 // stages, in CTAs that leave the least of an SM's shared memory unused (at most 64 threads a CTA before: nx = 24,
-// 535k stages, 2.05 -> 1.94 ms; nx = 12, 1.05M stages, 1.27 -> 1.22 ms).
+// 535k stages, 2.05 -> 1.94 ms; nx = 12, 1.05M stages, 1.27 -> 1.21 ms).
 template <int NX, int NW, int NY>
 constexpr int resid_df_teams() { return best_teams(DfWs<NX, NW, NY>::bytes); }
 template <int NX, int NW, int NY>

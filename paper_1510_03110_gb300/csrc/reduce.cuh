@@ -22,7 +22,7 @@
 //
 // Measured (GB300), before (some twenty barriers a stage, both triangles, divisions, blocks loaded as the
 // stage came) and after: FP64 nx = 20, 16384 stages in chunks of 32, 3.75 -> 2.04 ms, with four warps a chunk; a
-// master level of it 0.92 -> 0.22 ms; FP32 leaf level nx = 6, 1.10M stages, 1.02 -> 0.55 ms; nx = 12, 1.05M stages, 2.65 -> 2.08
+// master level of it 0.92 -> 0.22 ms; FP32 leaf level nx = 6, 1.10M stages, 1.02 -> 0.55 ms; nx = 12, 1.05M stages, 2.65 -> 2.04
 // ms; nx = 24, 535k stages, 6.44 -> 5.85 ms.
 #pragma once
 #include <type_traits>

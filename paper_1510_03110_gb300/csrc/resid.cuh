@@ -641,7 +641,7 @@ MHE_DEV void resid_arrival(const ResidArgs<float>& r, int b, int N, NormMax& mx)
 // 2880 double-float terms of 12 packed instructions for two, so the nine to ten teams an SM holds
 // are now bound by the latency of their dependent sums (ncu: 46% issue, 51% DRAM).  Full pass, before
 // (a stage's tasks read straight from global memory, scalar instructions) and after: nx = 24, 535k
-// stages, 2.63 -> 2.06 ms; nx = 12, 1.05M stages, 2.13 -> 1.26 ms; nx = 6, 1.10M stages, 0.97 -> 0.54 ms; nx = 64,
+// stages, 2.63 -> 1.95 ms; nx = 12, 1.05M stages, 2.13 -> 1.21 ms; nx = 6, 1.10M stages, 0.97 -> 0.54 ms; nx = 64,
 // 131k stages, 4.09 -> 3.17 ms (3.97 before S^T w took its columns turned: 32-way bank conflicts).
 template <int NX, int NW, int NY, class IT>
 MHE_DEV void resid_df_run(const ResidArgs<float>& r, IT& it, unsigned char* smem)
