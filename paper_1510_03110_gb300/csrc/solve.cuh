@@ -11,7 +11,8 @@
 // each a couple of microseconds of latency, and every allowed correction is
 // launched whether an instance still needs it or not.  For a batch of few or small
 // instances that is most of the solve: one estimate of nx = 12, N = 200 with 16 corrections
-// allowed took 213 launches and 0.81 ms, now 12 launches and 0.41 ms.
+// allowed took 213 launches and 0.81 ms; this launch brought it to 12 launches and 0.41 ms, and to 0.29 ms
+// with the reductions that came after it.
 #pragma once
 #include <cuda_runtime.h>
 #include <string.h>
