@@ -6,6 +6,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "device.h"
 #include "engine.h"
 #include "reduce_tc.cuh"
 #include "resid.cuh"
@@ -204,12 +205,11 @@ void launch_level_v(const LevelArgs<T>& a, void* stream)
         return;
     }
     const size_t smem = (size_t)W * op_count<T, NX, NW, UPPER, OP>() * sizeof(T);
-    static bool attr = false;
-    if (!attr) {
+    static OncePerDevice attr;
+    attr([&] {
         cudaFuncSetAttribute(k_level<T, NX, NW, UPPER, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        attr = true;
-    }
+    });
     const int grid = (a.nchunks + W - 1) / W;
     k_level<T, NX, NW, UPPER, OP><<<grid, MHE_TEAM * W, smem, (cudaStream_t)stream>>>(a);
 }
@@ -257,11 +257,10 @@ void launch_reduce_last(const LevelArgs<float>& a, int, void* stream)
     if (a.nchunks <= 0) return;
     constexpr size_t smem = (size_t)TcWs<NX, NW>::count * sizeof(float) + 16;
     static_assert(2 * (smem + 1024) <= 228 * 1024, "two CTAs per SM");
-    static bool attr = false;
-    if (!attr) {
+    static OncePerDevice attr;
+    attr([&] {
         cudaFuncSetAttribute(k_reduce_last<NX, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    });
     k_reduce_last<NX, NW><<<a.nchunks, MHE_TEAM, smem, (cudaStream_t)stream>>>(a);
 }
 
@@ -312,11 +311,10 @@ void launch_resid(const ResidArgs<TR>& r, void* stream)
         if (r.Ahi) {
             constexpr int W = resid_df_teams<NX, NW, NY>();
             constexpr size_t smem = (size_t)W * DfWs<NX, NW, NY>::bytes;
-            static bool attr = false;
-            if (!attr) {
+            static OncePerDevice attr;
+            attr([&] {
                 cudaFuncSetAttribute(k_resid_df<NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                attr = true;
-            }
+            });
             const long long blocks = (r.nstages + W - 1) / W;
             const long long room = (long long)device_sms() * resid_df_blocks<NX, NW, NY>();
             k_resid_df<NX, NW, NY><<<(unsigned)(blocks < room ? blocks : room), W * MHE_TEAM, smem,
@@ -354,11 +352,10 @@ void launch_prep(const PrepArgs& p, void* stream)
     if (p.nstages <= 0) return;
     constexpr int W = prep_warps<NX, NW, NY>();
     const size_t smem = (size_t)W * PrepSmem<NX, NW, NY>::count * 8;
-    static bool attr = false;
-    if (!attr) {
+    static OncePerDevice attr;
+    attr([&] {
         cudaFuncSetAttribute(k_prep<NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    });
     const long long grid = (p.nstages + W - 1) / W;
     k_prep<NX, NW, NY><<<(unsigned)grid, MHE_TEAM * W, smem, (cudaStream_t)stream>>>(p);
 }
@@ -414,11 +411,10 @@ void launch_assemble(long long S, const double* C, const double* R, const double
     if (S <= 0) return;
     constexpr int W = asm_warps<NX, NW, NY>();
     const size_t smem = (size_t)W * AsmSmem<NX, NW, NY>::count * 8;
-    static bool attr = false;
-    if (!attr) {
+    static OncePerDevice attr;
+    attr([&] {
         cudaFuncSetAttribute(k_assemble<NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    });
     const long long grid = (S + W - 1) / W;
     k_assemble<NX, NW, NY><<<(unsigned)grid, MHE_TEAM * W, smem, (cudaStream_t)stream>>>(S, C, R, yt, wt, Q, l, c);
 }

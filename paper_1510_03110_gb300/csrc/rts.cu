@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/mhe.h"
+#include "device.h"
 #include "tree.cuh"
 
 namespace mhe {
@@ -284,11 +285,10 @@ template <int NX, int NW, int NY>
 void launch_rts(const RtsArgs& r, void* stream)
 {
     const size_t smem = Ws<double, NX>::count * sizeof(double);
-    static bool attr = false;
-    if (!attr) {
+    static mhe::OncePerDevice attr;
+    attr([&] {
         cudaFuncSetAttribute(k_rts<NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    });
     k_rts<NX, NW, NY><<<r.batch, 32, smem, (cudaStream_t)stream>>>(r);
 }
 

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 #include <string.h>
 
+#include "device.h"
 #include "resid.cuh"
 #include "tree.cuh"
 
@@ -190,16 +191,16 @@ constexpr size_t solve_smem()
     return (size_t)solve_teams<T, NX, NW, NY>() * solve_words<T, NX, NW, NY>() * 8;
 }
 
-// clusters of more than eight CTAs and the shared memory, allowed once per kernel
+// clusters of more than eight CTAs and the shared memory, allowed once per kernel and GPU
 template <typename T, int NX, int NW, int NY>
 void solve_attributes()
 {
-    static bool attr = false;
-    if (attr) return;
-    cudaFuncSetAttribute(k_solve<T, NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)solve_smem<T, NX, NW, NY>());
-    cudaFuncSetAttribute(k_solve<T, NX, NW, NY>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    attr = true;
+    static OncePerDevice attr;
+    attr([] {
+        cudaFuncSetAttribute(k_solve<T, NX, NW, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)solve_smem<T, NX, NW, NY>());
+        cudaFuncSetAttribute(k_solve<T, NX, NW, NY>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
 }
 
 template <typename T, int NX, int NW, int NY>
@@ -226,7 +227,8 @@ void launch_solve(const SolveArgs<T>& p, void* stream)
 template <typename T, int NX, int NW, int NY>
 int solve_max_cluster()
 {
-    static const int most = [] {
+    static PerDevice most;
+    return most([] {
         solve_attributes<T, NX, NW, NY>();
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof(cfg));
@@ -239,13 +241,13 @@ int solve_max_cluster()
             c = 1;
         }
         return c < kSolveMaxCluster ? c : kSolveMaxCluster;
-    }();
-    return most;
+    });
 }
 
 inline int device_sms()
 {
-    static const int sms = [] {
+    static PerDevice sms;
+    return sms([] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
@@ -253,8 +255,7 @@ inline int device_sms()
             v = 152;
         }
         return v;
-    }();
-    return sms;
+    });
 }
 
 // CTAs per instance of a fused solve for a batch whose longest horizon is max_N, or 0 for a launch
