@@ -35,7 +35,7 @@ public:
     }
 };
 
-// a positive number looked up once per GPU
+// a number >= 0 looked up once per GPU (kept plus one: 0 is not looked up yet)
 class PerDevice {
     std::atomic<int> v_[kDeviceSlots] = {};
 
@@ -46,10 +46,10 @@ public:
         const int d = device_slot();
         if (d >= 0) {
             const int v = v_[d].load(std::memory_order_relaxed);
-            if (v > 0) return v;
+            if (v > 0) return v - 1;
         }
         const int v = f();
-        if (d >= 0) v_[d].store(v, std::memory_order_relaxed);
+        if (d >= 0) v_[d].store(v + 1, std::memory_order_relaxed);
         return v;
     }
 };

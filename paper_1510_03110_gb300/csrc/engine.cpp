@@ -719,7 +719,7 @@ bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0
     const bool fp64 = sizeof(T) == 8;
     const size_t L = lv.size();
     if (!has_fused(fp64)) return false;
-    const int cl = resume ? 4 : ops->solve_cluster(fp64, plan.batch, plan.max_N);
+    const int cl = resume ? 4 : ops->solve_cluster(fp64, mheC != nullptr, plan.batch, plan.max_N);
     if (cl < 1) return false;
     SolveArgs<T> p;
     memset(&p, 0, sizeof(p));

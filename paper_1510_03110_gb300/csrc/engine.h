@@ -53,9 +53,9 @@ struct ShapeOps {
     void (*solve64)(const SolveArgs<double>&, void* stream);
     void (*solve32)(const SolveArgs<float>&, void* stream);
     void (*solve_mhe32)(const SolveArgs<float>&, void* stream);
-    // CTAs per instance that solve takes for a batch whose longest horizon is max_N;
-    // 0: one launch per level pass is the faster way
-    int (*solve_cluster)(int fp64, int batch, int max_N);
+    // CTAs per instance that solve takes for a batch whose longest horizon is max_N (mhe: the MHE-form
+    // residual); 0: one launch per level pass is the faster way
+    int (*solve_cluster)(int fp64, int mhe, int batch, int max_N);
 };
 
 // The reductions of one shape with wider teams (levels with few chunks).

@@ -19,12 +19,11 @@
 
 #include "device.h"
 #include "resid.cuh"
+#include "solve_rule.h"
 #include "tree.cuh"
 
 namespace mhe {
 MHE_TEAM_NS_BEGIN
-
-constexpr int kSolveMaxCluster = 16;
 
 // 8-byte words of shared memory one team needs: the larger of the vector passes' workspaces and the residual's
 template <typename T, int NX, int NW, int NY>
@@ -223,27 +222,6 @@ void launch_solve(const SolveArgs<T>& p, void* stream)
     cudaLaunchKernelEx(&cfg, k_solve<T, NX, NW, NY>, p);
 }
 
-// The largest cluster of the kernel's CTAs this device can schedule, at most kSolveMaxCluster
-template <typename T, int NX, int NW, int NY>
-int solve_max_cluster()
-{
-    static PerDevice most;
-    return most([] {
-        solve_attributes<T, NX, NW, NY>();
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3(kSolveMaxCluster);
-        cfg.blockDim = dim3(solve_threads<T, NX, NW, NY>());
-        cfg.dynamicSmemBytes = solve_smem<T, NX, NW, NY>();
-        int c = 0;
-        if (cudaOccupancyMaxPotentialClusterSize(&c, k_solve<T, NX, NW, NY>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            c = 1;
-        }
-        return c < kSolveMaxCluster ? c : kSolveMaxCluster;
-    });
-}
-
 inline int device_sms()
 {
     static PerDevice sms;
@@ -258,24 +236,50 @@ inline int device_sms()
     });
 }
 
-// CTAs per instance of a fused solve for a batch whose longest horizon is max_N, or 0 for a launch
-// per level pass.  The clusters together about fill the chip once, and a team has at least about
-// one stage of the residual.  A team that would walk more than 16 stages per residual (six for nx > 12, whose
-// stages are longer), or a batch of more instances than SMs, keeps the chip busy with a launch per pass, which
-// spreads the chunks of all instances over all SMs.  Measured, launches per pass and fused: 79 instances of nx =
-// 12, N <= 160: 0.99 and 0.55 ms; one of nx = 12, N = 200: 0.36 and 0.29 ms; one of nx = 12, N = 1621 in FP64, 13 stages a
-// team: 0.85 and 0.82 ms; one of nx = 24, N = 1000, 8 stages a team: 0.85 and 0.96 ms; 256 of nx = 12, N <= 512: 1.32
-// and 2.17 ms; one of nx = 20, N = 16384 in FP64, 256 stages a team: 3.6 and 7 ms.
-template <int NX, int NW, int NY>
-int solve_cluster(int fp64, int batch, int max_N)
+// Clusters of 1 << i CTAs of the kernel the current GPU holds at a time, 0 for a size it cannot schedule
+template <typename T, int NX, int NW, int NY>
+int solve_resident(int i)
 {
-    const int teams = fp64 ? solve_teams<double, NX, NW, 0>() : solve_teams<float, NX, NW, NY>();
-    const int most = fp64 ? solve_max_cluster<double, NX, NW, 0>() : solve_max_cluster<float, NX, NW, NY>();
-    const int room = device_sms() * 11 / 10;
-    if (batch > room || most < 1) return 0;
-    int c = 1;
-    while (c * 2 <= most && batch * c * 2 <= room && (long long)c * 2 * teams * 10 <= (long long)max_N * 13) c *= 2;
-    return max_N <= (NX <= 12 ? 16 : 6) * c * teams ? c : 0;
+    static PerDevice most[kSolveSizes];
+    return most[i]([i] {
+        solve_attributes<T, NX, NW, NY>();
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(device_sms() * kSolveMaxCluster));
+        cfg.blockDim = dim3(solve_threads<T, NX, NW, NY>());
+        cfg.dynamicSmemBytes = solve_smem<T, NX, NW, NY>();
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1u << i;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_solve<T, NX, NW, NY>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        return n;
+    });
+}
+
+template <typename T, int NX, int NW, int NY>
+SolveRoom solve_room()
+{
+    SolveRoom r;
+    r.teams = solve_teams<T, NX, NW, NY>();
+    r.sms = device_sms();
+    for (int i = 0; i < kSolveSizes; ++i) r.resident[i] = solve_resident<T, NX, NW, NY>(i);
+    return r;
+}
+
+// CTAs per instance of a whole solve, or 0 (solve_rule.h); mhe: the residual is the double-float MHE form's
+template <int NX, int NW, int NY>
+int solve_cluster(int fp64, int mhe, int batch, int max_N)
+{
+    const SolveRoom r = fp64 ? solve_room<double, NX, NW, 0>()
+                             : (mhe ? solve_room<float, NX, NW, NY>() : solve_room<float, NX, NW, 0>());
+    return fused_cluster(NX, r, batch, max_N);
 }
 
 MHE_TEAM_NS_END

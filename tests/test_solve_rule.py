@@ -1,0 +1,78 @@
+"""When a solve runs as one launch (csrc/solve_rule.h), as plain arithmetic on the CPU: clusters that
+are all resident at a time, teams with work, horizons within the limit; a launch per pass otherwise."""
+import ctypes
+import os
+import shutil
+import subprocess
+import tempfile
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1510_03110_gb300", "csrc")
+
+SHIM = r'''
+#include "solve_rule.h"
+static mhe::SolveRoom room(int teams, int sms, const int* res)
+{
+    mhe::SolveRoom r;
+    r.teams = teams;
+    r.sms = sms;
+    for (int i = 0; i < mhe::kSolveSizes; ++i) r.resident[i] = res[i];
+    return r;
+}
+extern "C" int fused(int nx, int teams, int sms, const int* res, int batch, int N)
+{
+    return mhe::fused_cluster(nx, room(teams, sms, res), batch, N);
+}
+'''
+
+# clusters of 1, 2, 4, 8, 16 CTAs resident at a time: a GPU of 152 SMs in eight groups, one CTA an SM, and two
+RES1 = (152, 76, 36, 16, 4)
+RES2 = (304, 152, 72, 32, 14)
+TEAMS = {4: 32, 6: 32, 12: 16, 20: 8, 24: 8}
+
+
+@pytest.fixture(scope="module")
+def rule():
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    with tempfile.TemporaryDirectory() as d:
+        src, so = os.path.join(d, "s.cpp"), os.path.join(d, "s.so")
+        with open(src, "w") as f:
+            f.write(SHIM)
+        subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
+        L = ctypes.CDLL(so)
+        yield lambda name, nx, res, *a: getattr(L, name)(nx, TEAMS[nx], 152, (ctypes.c_int * 5)(*res), *a)
+
+
+def _limit(nx):
+    return 16 if nx <= 12 else 6
+
+
+@pytest.mark.parametrize("nx", sorted(TEAMS))
+@pytest.mark.parametrize("res", [RES1, RES2, (152, 76, 36, 0, 0), (152, 0, 0, 0, 0)])
+def test_one_launch_only_where_every_cluster_is_resident(rule, nx, res):
+    taken = 0
+    for batch in (1, 2, 4, 5, 8, 16, 17, 20, 36, 37, 76, 100, 152, 153, 167, 168, 400):
+        for N in (1, 2, 30, 100, 128, 200, 300, 400, 600, 800, 1000, 1600, 3000, 16384):
+            c = rule("fused", nx, res, batch, N)
+            if c == 0:
+                continue
+            taken += 1
+            assert c in (1, 2, 4, 8, 16)
+            assert batch <= res[(1, 2, 4, 8, 16).index(c)], (batch, N, c)
+            assert batch * c <= 167
+            assert N <= _limit(nx) * c * TEAMS[nx]
+            assert c == 1 or c * TEAMS[nx] * 10 <= N * 13   # a team has about a stage at least
+    assert taken > 20
+
+
+def test_measured_sides_of_the_line(rule):
+    # eight instances: clusters of 16 would take two waves (nx = 12, N = 800: 0.98 ms against 0.60)
+    assert rule("fused", 12, RES1, 8, 800) == 8
+    assert rule("fused", 12, RES1, 4, 800) == 16
+    assert rule("fused", 24, RES1, 20, 100) == 4
+    # long horizons: one launch per pass
+    assert rule("fused", 24, RES1, 1, 1000) == 0 and rule("fused", 20, RES1, 1, 16384) == 0
+    assert rule("fused", 12, RES1, 8, 3000) == 0 and rule("fused", 12, RES1, 256, 512) == 0
