@@ -704,7 +704,9 @@ constexpr int kPassRounds = 4;   // corrections launched pass by pass before the
 //
 // resume: a larger batch's last corrections.  Its passes are launched one by one for the first kPassRounds
 // corrections; what is left then is usually nothing or a few instances, and the corrections still allowed
-// would cost a dozen launches each: one launch takes them, whose clusters without work return at once.
+// would cost a dozen launches each: one launch takes them, whose clusters without work return at once.  Where the
+// instances that work on would make that much the slower way (few of them, long horizons: solve_rule.h), the
+// passes go on.
 bool Engine::has_fused(bool fp64) const
 {
     if (!ops->solve_cluster || !ordered || m64 || literal || mark_user || lv.size() > (size_t)kSolveLevels) return false;
@@ -719,7 +721,7 @@ bool Engine::solve_fused(const mhe_rhs* rhs, const T* l, const T* a, const T* x0
     const bool fp64 = sizeof(T) == 8;
     const size_t L = lv.size();
     if (!has_fused(fp64)) return false;
-    const int cl = resume ? 4 : ops->solve_cluster(fp64, mheC != nullptr, plan.batch, plan.max_N);
+    const int cl = (resume ? ops->resume_cluster : ops->solve_cluster)(fp64, mheC != nullptr, plan.batch, plan.max_N);
     if (cl < 1) return false;
     SolveArgs<T> p;
     memset(&p, 0, sizeof(p));

@@ -56,6 +56,8 @@ struct ShapeOps {
     // CTAs per instance that solve takes for a batch whose longest horizon is max_N (mhe: the MHE-form
     // residual); 0: one launch per level pass is the faster way
     int (*solve_cluster)(int fp64, int mhe, int batch, int max_N);
+    // the same for a larger batch's last corrections
+    int (*resume_cluster)(int fp64, int mhe, int batch, int max_N);
 };
 
 // The reductions of one shape with wider teams (levels with few chunks).

@@ -473,10 +473,11 @@ ShapeEntry make_shape()
         e.ops.solve32 = &launch_solve<float, NX, NW, 0>;
         e.ops.solve_mhe32 = &launch_solve<float, NX, NW, NY>;
         e.ops.solve_cluster = &solve_cluster<NX, NW, NY>;
+        e.ops.resume_cluster = &resume_cluster<NX, NW, NY>;
     } else {
         e.ops.solve64 = nullptr;
         e.ops.solve32 = e.ops.solve_mhe32 = nullptr;
-        e.ops.solve_cluster = nullptr;
+        e.ops.solve_cluster = e.ops.resume_cluster = nullptr;
     }
     e.ny = NY;
     e.assemble = &launch_assemble<NX, NW, NY>;

@@ -273,13 +273,24 @@ SolveRoom solve_room()
     return r;
 }
 
-// CTAs per instance of a whole solve, or 0 (solve_rule.h); mhe: the residual is the double-float MHE form's
+// the kernel a solve takes; mhe: the residual is the double-float MHE form's
+template <int NX, int NW, int NY>
+SolveRoom solve_room_of(int fp64, int mhe)
+{
+    if (fp64) return solve_room<double, NX, NW, 0>();
+    return mhe ? solve_room<float, NX, NW, NY>() : solve_room<float, NX, NW, 0>();
+}
+
+// CTAs per instance of a whole solve, and of a larger batch's last corrections, or 0 (solve_rule.h)
 template <int NX, int NW, int NY>
 int solve_cluster(int fp64, int mhe, int batch, int max_N)
 {
-    const SolveRoom r = fp64 ? solve_room<double, NX, NW, 0>()
-                             : (mhe ? solve_room<float, NX, NW, NY>() : solve_room<float, NX, NW, 0>());
-    return fused_cluster(NX, r, batch, max_N);
+    return fused_cluster(NX, solve_room_of<NX, NW, NY>(fp64, mhe), batch, max_N);
+}
+template <int NX, int NW, int NY>
+int resume_cluster(int fp64, int mhe, int batch, int max_N)
+{
+    return resumed_cluster(NX, solve_room_of<NX, NW, NY>(fp64, mhe), batch, max_N);
 }
 
 MHE_TEAM_NS_END

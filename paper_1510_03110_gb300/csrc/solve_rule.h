@@ -43,4 +43,25 @@ inline int fused_cluster(int nx, const SolveRoom& r, int batch, int max_N)
     return max_N <= solve_stages(nx) * c * r.teams ? c : 0;
 }
 
+// CTAs per instance of a larger batch's corrections after the first four, in one launch, or 0 to go on with a launch
+// per pass.  A solve that has converged by then (the usual one) saves the empty passes of every correction still
+// allowed; one that has not should not pay much for it, whether one instance works on or all do: one CTA, or two,
+// which is as far as the few chunks of an instance keep the teams busy.  Measured, twelve corrections allowed,
+// passes and clusters of 1, 2, 4, with none, a few and all instances working on after the fourth:
+//   MHE form, 1024 of nx = 6, N <= 2048:  4.11  3.74 3.74 3.75;  7.43  6.76 6.69 6.70;  16.2  19.0 20.7 28.8
+//   MHE form, 200 of nx = 12, N <= 300:   1.03  0.73 0.73 0.73;  1.50  1.23 1.21 1.21;   2.5   3.5  3.7  5.6
+//   Q form, 500 of nx = 4, N <= 512:      1.03  0.65 0.65 0.65;  1.68  1.44 1.38 1.35;   3.0   3.3  4.4  6.5
+//   Q form, 256 of nx = 12, N <= 512:     1.31  0.92 0.92 0.93;  2.48  2.23 2.15 2.11;   4.7   7.5  7.4  9.6
+// Left to the passes: few instances or long horizons (16 corrections used: one of nx = 20, N = 16384, 5.1 by passes
+// and 55 resumed with four CTAs; one of nx = 24, N = 2000 2.8 and 9.6), horizons with fewer chunks than teams (2000
+// of nx = 4, N <= 60: all 1.8 and 3.6), and above nx = 8 large batches (1024 of nx = 12, N <= 512: none 3.1 and
+// 2.8, all 11.2 and 18.9).
+inline int resumed_cluster(int nx, const SolveRoom& r, int batch, int max_N)
+{
+    if (2 * batch < r.sms || max_N < 4 * r.teams || (nx > 8 && batch > 2 * r.sms)) return 0;
+    const int most = (nx <= 8 ? 32 : solve_stages(nx)) * r.teams;   // stages of one CTA
+    if (r.resident[0] > 0 && max_N <= most) return 1;
+    return r.resident[1] > 0 && max_N <= 2 * most ? 2 : 0;
+}
+
 }  // namespace mhe

@@ -70,6 +70,24 @@ def test_last_corrections_in_one_launch(n, m, form, tol):
     assert a[1]["refine_iters"].max() > 5   # past the change-over
 
 
+@pytest.mark.parametrize("form", ["solve", "estimate"])
+@pytest.mark.parametrize("n,m,Ns,resumed", [
+    (6, 3, [2 + (37 * i) % 290 for i in range(180)], True),
+    (12, 6, [2 + (37 * i) % 290 for i in range(180)], True),
+    (20, 10, [2 + (7 * i) % 60 for i in range(200)], True),
+    (20, 10, [1500], False), (24, 12, [900, 5], False),                 # a long horizon, alone or nearly
+    (12, 6, [2 + (37 * i) % 290 for i in range(320)], False)])          # many instances of longer stages
+def test_late_corrections_take_the_route_of_the_rule(n, m, Ns, resumed, form):
+    """More than four corrections: the rest in one launch, or pass by pass to the end; equal bits either way."""
+    insts = [synth.mhe_instance(4400 + i % 40, n, m, m, N) for i, N in enumerate(Ns)]
+    d = device_inputs(insts)
+    a = _run(d, form, mhe.MHE_FP32_IR, False, refine_tol=1e-30, max_refine=9)
+    b = _run(d, form, mhe.MHE_FP32_IR, True, refine_tol=1e-30, max_refine=9)
+    _same(a, b)
+    assert a[1]["refine_iters"].max() == 9
+    assert (a[2] < b[2]) if resumed else (a[2] == b[2]), (a[2], b[2])
+
+
 @pytest.mark.parametrize("n,m", [(4, 2), (6, 3), (12, 6), (20, 10), (24, 12)])
 @pytest.mark.parametrize("prec,tol", [(mhe.MHE_FP64, 1e-10), (mhe.MHE_FP32_IR, 1e-8)])
 def test_levels_of_many_chunks(n, m, prec, tol):

@@ -24,6 +24,10 @@ extern "C" int fused(int nx, int teams, int sms, const int* res, int batch, int 
 {
     return mhe::fused_cluster(nx, room(teams, sms, res), batch, N);
 }
+extern "C" int resumed(int nx, int teams, int sms, const int* res, int batch, int N)
+{
+    return mhe::resumed_cluster(nx, room(teams, sms, res), batch, N);
+}
 '''
 
 # clusters of 1, 2, 4, 8, 16 CTAs resident at a time: a GPU of 152 SMs in eight groups, one CTA an SM, and two
@@ -76,3 +80,31 @@ def test_measured_sides_of_the_line(rule):
     # long horizons: one launch per pass
     assert rule("fused", 24, RES1, 1, 1000) == 0 and rule("fused", 20, RES1, 1, 16384) == 0
     assert rule("fused", 12, RES1, 8, 3000) == 0 and rule("fused", 12, RES1, 256, 512) == 0
+
+
+@pytest.mark.parametrize("nx", sorted(TEAMS))
+@pytest.mark.parametrize("res", [RES1, RES2, (152, 0, 0, 0, 0)])
+def test_late_corrections_in_one_launch_only_where_it_cannot_cost_much(rule, nx, res):
+    taken = 0
+    for batch in (1, 2, 8, 40, 75, 76, 100, 152, 200, 256, 304, 305, 512, 1024, 4096):
+        for N in (1, 8, 16, 31, 36, 60, 64, 96, 128, 200, 256, 300, 512, 1000, 2000, 2048, 4096, 16384):
+            c = rule("resumed", nx, res, batch, N)
+            if c == 0:
+                continue
+            taken += 1
+            assert c == 1 or (c == 2 and res[1] and N > (32 if nx <= 8 else _limit(nx)) * TEAMS[nx])
+            assert 2 * batch >= 152                                       # not a few long instances
+            assert N <= (32 if nx <= 8 else _limit(nx)) * c * TEAMS[nx]   # a straggler's share
+            assert N >= 4 * TEAMS[nx]                                     # teams with chunks
+            assert nx <= 8 or batch <= 304
+    assert taken > 0
+
+
+def test_measured_sides_of_the_resumed_line(rule):
+    # a long horizon, alone or few: the passes (one of nx = 20, N = 16384: 5.1 ms, resumed 55)
+    assert rule("resumed", 20, RES1, 1, 16384) == 0 and rule("resumed", 24, RES1, 1, 2000) == 0
+    assert rule("resumed", 24, RES1, 512, 2048) == 0 and rule("resumed", 12, RES1, 1024, 512) == 0
+    assert rule("resumed", 4, RES1, 2000, 60) == 0
+    # a bank of short horizons, a large batch of small states
+    assert rule("resumed", 12, RES1, 256, 512) == 2 and rule("resumed", 6, RES1, 1024, 2048) == 2
+    assert rule("resumed", 4, RES1, 500, 512) == 1
