@@ -578,10 +578,12 @@ struct StageStride {
     }
 };
 
-// running maxima of |r| (float bits), |z|, |b| (double bits) of one instance, merged into its norms at once
+// running maxima of |r| (float bits of the double-float rows, double bits of the FP64 ones), |z|, |b| (double bits)
+// of one instance, merged into its norms at once
 struct NormMax {
     unsigned r = 0;
-    unsigned long long z = 0, b = 0;
+    unsigned long long rd = 0, z = 0, b = 0;
+    MHE_DEV void see_rd(double v) { const unsigned long long u = abs_bits(v); rd = u > rd ? u : rd; }
     MHE_DEV void see_r(float v) { const unsigned u = __float_as_uint(v) & 0x7fffffffu; r = u > r ? u : r; }
     MHE_DEV void see_z(double v) { const unsigned long long u = abs_bits(v); z = u > z ? u : z; }
     MHE_DEV void see_b(double v) { const unsigned long long u = abs_bits(v); b = u > b ? u : b; }
@@ -590,7 +592,8 @@ struct NormMax {
         constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32;
         const unsigned mask =
             CW == 32 ? 0xffffffffu : (((1u << CW) - 1u) << ((threadIdx.x & 31) & ~(CW - 1)));
-        unsigned long long m[3] = {abs_bits(f64_of(__uint_as_float(r))), z, b};
+        const unsigned long long rf = abs_bits(f64_of(__uint_as_float(r)));
+        unsigned long long m[3] = {rf > rd ? rf : rd, z, b};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
 #pragma unroll
@@ -601,7 +604,7 @@ struct NormMax {
             if ((lane_id() & (CW - 1)) == 0 && m[k]) atomic_max_u64(norms + k, m[k]);
         }
         r = 0;
-        z = b = 0;
+        rd = z = b = 0;
     }
 };
 
@@ -617,17 +620,17 @@ MHE_DEV void resid_arrival(const ResidArgs<float>& r, int b, int N, NormMax& mx)
         double q = ln;
 #pragma unroll 4
         for (int j = 0; j < NX; ++j) q = fma(P0[i + j * NX], wt[j], q);
-        const float rx = f32_rn(ln - l), rw = f32_rn(q), rd = f32_rn(x + w - xn), ri = f32_rn(x0 - x);
-        r.rl0[(long long)b * 2 * NX + i] = rx;
-        r.rl0[(long long)b * 2 * NX + NX + i] = rw;
-        r.ra0[(long long)b * NX + i] = rd;
-        r.rx0[(long long)b * NX + i] = ri;
-        mx.see_r(rx); mx.see_r(rw); mx.see_r(rd); mx.see_r(ri);
+        const double rx = ln - l, rd = x + w - xn, ri = x0 - x;
+        r.rl0[(long long)b * 2 * NX + i] = f32_rn(rx);
+        r.rl0[(long long)b * 2 * NX + NX + i] = f32_rn(q);
+        r.ra0[(long long)b * NX + i] = f32_rn(rd);
+        r.rx0[(long long)b * NX + i] = f32_rn(ri);
+        mx.see_rd(rx); mx.see_rd(q); mx.see_rd(rd); mx.see_rd(ri);
         mx.see_z(x); mx.see_z(l); mx.see_z(w);
         mx.see_b(x0);
         if (N == 1) {   // terminal rows: -(0 - lambda_N)
             r.rlN[(long long)b * NX + i] = f32_rn(-ln);
-            mx.see_r(f32_rn(ln));
+            mx.see_rd(ln);
             mx.see_z(xn); mx.see_z(ln);
         }
     });
