@@ -174,22 +174,20 @@ struct Addr {
     }
 };
 
-// L2 prefetch of the blocks of level-0 stage t of instance b (t >= 1) a pass
-// reads: PF_A, PF_B, PF_Q, PF_L (l) and PF_AV (a) select them
-enum { PF_A = 1, PF_B = 2, PF_Q = 4, PF_L = 8, PF_AV = 16, PF_ALL = 31 };
+// L2 prefetch of A, B, Q, l and a of level-0 stage t of instance b (t >= 1)
 template <typename T, int NX, int NW>
-MHE_DEV void prefetch_leaf(const LevelArgs<T>& a, int b, int t, int what = PF_ALL)
+MHE_DEV void prefetch_leaf(const LevelArgs<T>& a, int b, int t)
 {
     if (t < 1) return;
 #ifdef MHE_BOUNDS_CHECK
     if (!in_ext(a.in_off[b] + t - 1, a.ext_S_in) || !in_ext(a.rhs_off[b] + t - 1, a.ext_S_in)) return;
 #endif
     const long long s = a.in_off[b] + t - 1;
-    if (what & PF_A) prefetch_l2(a.A + s * NX * NX, (int)(sizeof(T) * NX * NX));
-    if (what & PF_B) prefetch_l2(a.B + s * NX * NW, (int)(sizeof(T) * NX * NW));
-    if (what & PF_Q) prefetch_l2(a.Q + s * (NX + NW) * (NX + NW), (int)(sizeof(T) * (NX + NW) * (NX + NW)));
-    if ((what & PF_L) && a.l) prefetch_l2(a.l + (a.rhs_off[b] + t - 1) * (NX + NW), (int)(sizeof(T) * (NX + NW)));
-    if ((what & PF_AV) && a.a) prefetch_l2(a.a + (a.rhs_off[b] + t - 1) * NX, (int)(sizeof(T) * NX));
+    prefetch_l2(a.A + s * NX * NX, (int)(sizeof(T) * NX * NX));
+    prefetch_l2(a.B + s * NX * NW, (int)(sizeof(T) * NX * NW));
+    prefetch_l2(a.Q + s * (NX + NW) * (NX + NW), (int)(sizeof(T) * (NX + NW) * (NX + NW)));
+    if (a.l) prefetch_l2(a.l + (a.rhs_off[b] + t - 1) * (NX + NW), (int)(sizeof(T) * (NX + NW)));
+    if (a.a) prefetch_l2(a.a + (a.rhs_off[b] + t - 1) * NX, (int)(sizeof(T) * NX));
 }
 
 MHE_TEAM_NS_END

@@ -86,12 +86,11 @@ MHE_DEV void load_AB(Ws<T, NX>& s, const StageRef<T>& st)
 }
 
 // Store the R x C column-major block at src (shared memory, leading dimension
-// LD) to dst (global, leading dimension R), times sgn, keeping only i >= j when
-// LOWER; then tail(k) for k < ntail in the same step.  FP32 blocks of a multiple
-// of four rows go in 16-byte pieces (every column of dst then starts 16-byte
-// aligned, as dst does: the stored blocks are laid out back to back in a 256-byte
-// aligned arena), others element by element.
-template <typename T, int R, int C, int LD, bool LOWER = false, class TF>
+// LD) to dst (global, leading dimension R), times sgn; then tail(k) for k < ntail in the
+// same step.  FP32 blocks of a multiple of four rows go in 16-byte pieces (every
+// column of dst then starts 16-byte aligned, as dst does: the stored blocks are laid out
+// back to back in a 256-byte aligned arena), others element by element.
+template <typename T, int R, int C, int LD, class TF>
 MHE_DEV void store_block(T* dst, const T* src, T sgn, int ntail, TF&& tail)
 {
     if constexpr (sizeof(T) == 4 && R % 4 == 0 && LD % 4 == 0) {
@@ -105,7 +104,7 @@ MHE_DEV void store_block(T* dst, const T* src, T sgn, int ntail, TF&& tail)
             float v[4];
             ld16(src + i + j * LD, v);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = (LOWER && i + q < j) ? 0.f : sgn * v[q];
+            for (int q = 0; q < 4; ++q) v[q] = sgn * v[q];
             st16(dst + i + j * R, v);
         });
     } else {
@@ -115,7 +114,7 @@ MHE_DEV void store_block(T* dst, const T* src, T sgn, int ntail, TF&& tail)
                 return;
             }
             const int i = r % R, j = r / R;
-            dst[r] = (LOWER && i < j) ? (T)0 : sgn * src[i + j * LD];
+            dst[r] = sgn * src[i + j * LD];
         });
     }
 }

@@ -142,12 +142,12 @@ MHE_DEV void ldv(const T* p, T (&v)[V])
 template <int K, typename T>
 MHE_DEV T coldot(const T* col, const T* v, T init)
 {
-    constexpr int V = vec_of<T>(K), KV = K;
+    constexpr int V = vec_of<T>(K);
     T acc[V];
 #pragma unroll
     for (int q = 0; q < V; ++q) acc[q] = (T)0;
 #pragma unroll
-    for (int p = 0; p < KV; p += V) {
+    for (int p = 0; p < K; p += V) {
         T a[V], b[V];
         ldv(col + p, a);
         ldv(v + p, b);
@@ -164,12 +164,12 @@ MHE_DEV T coldot(const T* col, const T* v, T init)
 template <int K, int LD, typename T>
 MHE_DEV T rowdot(const T* row, const T* v, T init)
 {
-    constexpr int V = vec_of<T>(K), KV = K;
+    constexpr int V = vec_of<T>(K);
     T acc[V];
 #pragma unroll
     for (int q = 0; q < V; ++q) acc[q] = (T)0;
 #pragma unroll
-    for (int p = 0; p < KV; p += V) {
+    for (int p = 0; p < K; p += V) {
         T b[V];
         ldv(v + p, b);
 #pragma unroll
