@@ -129,7 +129,7 @@ struct LevelBuf {   // every array of the level's compute type (FP64 at k >= 1 w
 // Serving with reuse: the stored factors of every level and the master-stage data
 // of the levels k >= 1 live in stores the server keeps across rounds (one ring
 // per estimator and level, addressed through the chunk descriptors), not in a
-// context's workspace.  Per level: P, L^{-T} of G = L L^T, K, k, L; A^, R^T, Q^_x, a^, l^_x.
+// context's workspace.  Per level: P, the factor of G, K, k, L; A^, R^T, Q^_x, a^, l^_x.
 struct ExtStores {
     std::vector<void*> Pst, Lgst, Kst, kst, Lst, Ah, Bh, Qxh, ah, lxh;
     size_t levels() const { return Pst.size(); }

@@ -28,9 +28,9 @@ namespace {
 constexpr long long kScratchDoubles = 1LL << 20;
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
 
-// doubles of scratch one call needs: per stage t >= 1 the Cholesky factor of
-// G (nw^2), K (nw x nx) and k (nw); for the arrival stage the same with
-// width nx
+// doubles of scratch one call is allowed: per stage t >= 1 a factor of G (nw^2), K (nw x nx) and k (nw); for the
+// arrival stage the same with width nx.  The solve needs no stored factor of G (it has one right-hand side, carried
+// along), so the kernel lays out K and k only; the limit is the documented one
 long long scratch_need(int nx, int nw, int N)
 {
     return (long long)N * ((long long)nw * nw + (long long)nw * nx + nw) + 2LL * nx * nx + nx;
@@ -68,10 +68,8 @@ __global__ void __launch_bounds__(32) k_serial_noalloc(int N, const double* A, c
     g.w_off = &off[1];
     g.l = l; g.a = a; g.x0 = x0;
     double* p = scratch;
-    g.Lgst = p; p += (long long)N * NW * NW;
     g.Kst = p; p += (long long)N * NW * NX;
     g.kst = p; p += (long long)N * NW;
-    g.Lgst0 = p; p += NX * NX;
     g.Kst0 = p; p += NX * NX;
     g.kst0 = p;
     g.status = st;

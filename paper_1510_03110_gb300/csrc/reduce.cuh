@@ -6,11 +6,12 @@
 //   2. W^T P W + Q, whose blocks are F, H and G (symmetric: one triangle);  W^T u
 //   3. G = L L^T, and beside it A^T V
 //   4. per column, in registers: Y = L^{-1} H^T, y = L^{-1} g, Z = L^{-1} BV and from them
-//      K = -L^{-T} Y, k = L^{-T} y, L_t = -L^{-T} Z, straight to global memory; L^{-1}
+//      K = -L^{-T} Y, k = L^{-T} y, L_t = -L^{-T} Z, straight to global memory, as L itself
 //   5. P <- F - Y^T Y,  V <- A^T V - Y^T Z,  Q^_w += Z^T Z,
 //      Psi <- A^T u - l_x - Y^T y,  v <- v + V^T a + Z^T y
 // (K^T B^T V = -Y^T Z and V^T (a + B k) = V^T a + Z^T y, so K, k and L_t are only stored.)
-// Five team barriers a stage; the next stage's A, B and a are copied asynchronously from
+// Six team barriers a stage (one after each step, one once the stage's copies have landed), and in FP64 one more
+// per pivot column of G while a single team factors it; the next stage's A, B and a are copied asynchronously from
 // the end of step 3 on.
 //
 // What bounds it.  FP64: an instruction of a warp costs 64 cycles of its SM quarter whatever
@@ -360,14 +361,28 @@ MHE_DEV int chol_pivoted(T* Gm, double rank_rel, T* permv, T* sc)
     return (int)sc[3];
 }
 
+// The factor in G (columns LD apart) to dst, columns MT apart; whatever lies above the diagonal goes with it
+template <typename T, int MT, int LD>
+MHE_DEV void store_factor(T* dst, const T* G)
+{
+    if constexpr (sizeof(T) == 4 && MT % 4 == 0 && LD % 4 == 0) {
+        each<MT * MT / 4>([&](int u) {
+            const int i = 4 * (u % (MT / 4)), j = u / (MT / 4);
+            st16(dst + 4 * u, ld16g(G + i + j * LD));
+        });
+    } else {
+        each<MT * MT>([&](int r) { dst[r] = G[r % MT + (r / MT) * LD]; });
+    }
+}
+
 // Step 4: one column per lane (or per pair of lanes, H = 2, each holding every other row) through both
-// substitutions.  Columns 0 .. n-1: H^T -> Y, K; n: g -> y, k; then BV -> Z, L_t; then the unit vectors -> L^{-1}.
+// substitutions.  Columns 0 .. n-1: H^T -> Y, K; n: g -> y, k; then BV -> Z, L_t.
 template <typename T, int NX, int MT, int LM, int H>
-MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* Lgout, T* Kout, T* kout, T* Lout)
+MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* Kout, T* kout, T* Lout)
 {
     constexpr int MH = (MT + H - 1) / H, VK = vec_of<T>(MT);
     static_assert(MT % VK == 0 && LM % VK == 0, "whole vectors of a column");
-    const int nz = want_v ? NX : 0, nc = NX + 1 + nz + (Lgout ? MT : 0);
+    const int nc = NX + 1 + (want_v ? NX : 0);
     const int half = H == 1 ? 0 : (lane_id() & 1);
     const unsigned mask = H == 1 ? 0u : 0xffffffffu;
     (void)mask;
@@ -375,14 +390,13 @@ MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* L
     for (int c0 = 0; c0 < nc; c0 += MHE_TEAM / H) {
         const int c = c0 + lane_id() / H;
         const bool on = c < nc;
-        const bool unit = c >= NX + 1 + nz, zc = !unit && c > NX;
-        const int uc = c - (NX + 1 + nz);
-        T* col = unit || !on ? nullptr : (zc ? Z + (c - NX - 1) * LM : Y + c * LM);
+        const bool zc = c > NX;
+        T* col = !on ? nullptr : (zc ? Z + (c - NX - 1) * LM : Y + c * LM);
         T y[MH];
         if constexpr (H == 1) {
             if (!on) continue;
 #pragma unroll
-            for (int i = 0; i < MT; ++i) y[i] = unit ? (T)(i == uc ? 1 : 0) : col[i];
+            for (int i = 0; i < MT; ++i) y[i] = col[i];
 #pragma unroll
             for (int i = 0; i < MT; ++i) {
                 T a[2] = {y[i], (T)0};
@@ -395,11 +409,6 @@ MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* L
                         if (p + q < i) a[q & 1] -= l[q] * y[p + q];
                 }
                 y[i] = (a[0] + a[1]) * R[i + i * LM];
-            }
-            if (unit) {
-#pragma unroll
-                for (int i = 0; i < MT; ++i) Lgout[uc + i * MT] = y[i];
-                continue;
             }
 #pragma unroll
             for (int i = 0; i < MT; ++i) col[i] = y[i];
@@ -425,7 +434,7 @@ MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* L
 #pragma unroll
             for (int q = 0; q < MH; ++q) {
                 const int i = 2 * q + half;
-                y[q] = !on || i >= MT ? (T)0 : (unit ? (T)(i == uc ? 1 : 0) : col[i]);
+                y[q] = on && i < MT ? col[i] : (T)0;
             }
 #pragma unroll
             for (int p = 0; p < MT; ++p) {
@@ -440,10 +449,7 @@ MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* L
 #pragma unroll
             for (int q = 0; q < MH; ++q) {
                 const int i = 2 * q + half;
-                if (on && i < MT) {
-                    if (unit) Lgout[uc + i * MT] = y[q];
-                    else col[i] = y[q];
-                }
+                if (on && i < MT) col[i] = y[q];
             }
 #pragma unroll
             for (int p = MT - 1; p >= 0; --p) {
@@ -455,7 +461,7 @@ MHE_DEV void solve_columns(T* Y, T* Z, const T* G, const T* R, bool want_v, T* L
                     else if (i == p) y[q] = f;
                 }
             }
-            T* dst = unit || !on ? nullptr : (zc ? (Lout ? Lout + (c - NX - 1) * MT : nullptr) : (c < NX ? Kout + c * MT : kout));
+            T* dst = !on ? nullptr : (zc ? (Lout ? Lout + (c - NX - 1) * MT : nullptr) : (c < NX ? Kout + c * MT : kout));
 #pragma unroll
             for (int q = 0; q < MH; ++q) {
                 const int i = 2 * q + half;
@@ -597,7 +603,8 @@ MHE_DEV bool reduce_stage(RedPtr<T>& s, const StageRef<T>& st, T* Pout, T* Lgout
     const bool bad = *s.flag != (T)0;
     // 4.
     constexpr int H = sizeof(T) == 8 && TL >= 128 ? 2 : 1;
-    solve_columns<T, NX, MT, lm, H>(s.Y, s.Z, s.G, s.R, want_v, Lgout, Kout, kout, Lout);
+    if (Lgout) store_factor<T, MT, lm>(Lgout, s.G);
+    solve_columns<T, NX, MT, lm, H>(s.Y, s.Z, s.G, s.R, want_v, Kout, kout, Lout);
     wsync();
     // 5. (the arrival stage: A^T V = V, F = P)
     const T* y = s.Y + NX * lm;
@@ -694,11 +701,11 @@ MHE_DEV void reduce_chunk_small(const LevelArgs<T>& a, int ci, T* smem)
             r.R = s.X;
             bad = reduce_stage<T, NX, NX, KIND_ARRIVAL>(
                 r, Addr<T, NX, NW>::arrival(a, b), a.store_P ? a.Pst0 + (long long)b * NX * NX : nullptr,
-                a.Lgst0 + (long long)b * NX * NX, a.Kst0 + (long long)b * NX * NX, a.kst0 + (long long)b * NX,
+                a.Lgst0 ? a.Lgst0 + (long long)b * NX * NX : nullptr, a.Kst0 + (long long)b * NX * NX, a.kst0 + (long long)b * NX,
                 last ? nullptr : a.Lst0 + (long long)b * NX * NX, !last, a.piv_rel, [] {});
         } else {
             bad = reduce_stage<T, NX, MT, KIND>(s, ref(tt), a.store_P ? a.Pst + g * NX * NX : nullptr,
-                                                a.Lgst + g * MT * MT, a.Kst + g * MT * NX, a.kst + g * MT,
+                                                a.Lgst ? a.Lgst + g * MT * MT : nullptr, a.Kst + g * MT * NX, a.kst + g * MT,
                                                 last ? nullptr : a.Lst + g * MT * NX, !last, a.piv_rel,
                                                 [&] { load(tt - 1); });
         }

@@ -213,8 +213,8 @@ MHE_DEV void reduce_last_tc(const LevelArgs<float>& a, int ci, float* sm, TcStat
             factor_block<float, NW, lm, MHE_TEAM>(G, R, tmp, a.piv_rel, sc);
             wsync();
             bad = sc[0] != 0.f;
-            solve_columns<float, NX, NW, lm, 1>(Y, Y, G, R, false, a.Lgst + gs * NW * NW, a.Kst + gs * NW * NX,
-                                                a.kst + gs * NW, nullptr);
+            store_factor<float, NW, lm>(a.Lgst + gs * NW * NW, G);
+            solve_columns<float, NX, NW, lm, 1>(Y, Y, G, R, false, a.Kst + gs * NW * NX, a.kst + gs * NW, nullptr);
             wsync();
             prod<float, NX, NX, NW, lm, lm, true, 0, MHE_TEAM>(
                 Y, Y, [](int, int) { return None(); }, [&](int i, int j, float v, None) {
@@ -232,7 +232,6 @@ MHE_DEV void reduce_last_tc(const LevelArgs<float>& a, int ci, float* sm, TcStat
             s.PB = sm + W::aY;
             s.K = s.H = sm + W::aK;
             s.Psi = Psi; s.g = g; s.k = e; s.tmp = tmp; s.sc = sc; s.tv = tv;
-            float* const l64 = a.Lgst0 + (long long)b * NX * NX;
             each<NX>([&](int i) {
                 tv[i] = Psi[i];
                 for (int p = 0; p < NX; ++p) tv[i] -= P[i + p * ld] * XA::a(st, p);
@@ -257,7 +256,7 @@ MHE_DEV void reduce_last_tc(const LevelArgs<float>& a, int ci, float* sm, TcStat
             store_block<float, NX, NX, ld>(a.Kst0 + (long long)b * NX * NX, s.K, 1.f, NX,
                                            [&](int j) { a.kst0[(long long)b * NX + j] = e[j]; });
             // nothing reads P_0, Psi_0: no problem lies above, and x_0 is known
-            store_inverse<float, NX, NX>(s, l64);
+            store_factor<float, NX, ld>(a.Lgst0 + (long long)b * NX * NX, s.G);
         }
         if (bad && bad_t < 0) bad_t = t;
     }

@@ -298,7 +298,7 @@ void eff_plan(const mhe_server* s, int nx, int nw, int* leaf, int* br, int* top)
     *top = s->top_len > 0 ? s->top_len : 4;
 }
 
-// elements of one store slot at level k: P, L^{-T} of G = L L^T, K, k, L (and at k >= 1 the
+// elements of one store slot at level k: P, the factor of G, K, k, L (and at k >= 1 the
 // master stage A^, R^T, Q^_x, a^, l^_x)
 size_t slot_elems(int k, int n, int m)
 {

@@ -282,21 +282,6 @@ MHE_DEV void col_solves(const Ws<T, NX>& s, bool upper, FR&& rhs, FY&& putY, FX&
     });
 }
 
-// L^{-1} of the factor in s.G to dst, transposed (entry (q, j) of the M x M column-major block is
-// L^{-1}(j, q), zero for q > j): the vector passes apply it as two products
-template <typename T, int NX, int M>
-MHE_DEV void store_inverse(Ws<T, NX>& s, T* dst)
-{
-    constexpr int ld = Ws<T, NX>::ld;
-    lower_solve<T, NX, M, M>(s, [&](int i, int c) -> T { return (T)(i == c ? 1 : 0); },
-                             [&](int i, int c) -> T { return s.H[i + c * ld]; },
-                             [&](int i, int c, T v) { s.H[i + c * ld] = v; });
-    wfor(M * M, [&](int r) {
-        const int c = r % M, i = r / M;
-        dst[r] = i >= c ? s.H[i + c * ld] : (T)0;
-    });
-}
-
 // ---- the stage products on the tensor cores (tcgen05, kind::tf32) -------------
 //
 // Tensor state of a team whose stage products run on the tensor cores: TMEM
@@ -672,7 +657,7 @@ MHE_DEV void tc_stage_products_bf16(Ws<float, NX>& s, const StageRef<float>& st,
 
 // One backward stage of Algorithm 4 (or Algorithms 1-2 when want_v is false).
 // On entry s.P = P_{t+1}, s.Psi = Psi_{t+1}, s.V = V_{t+1}, s.v = v_{t+1},
-// s.Qw = partial Q^_w.  Stores P_{t+1}, L^{-T} of G_{t+1} = L L^T, K_{t+1}, k_{t+1},
+// s.Qw = partial Q^_w.  Stores P_{t+1}, L of G_{t+1} = L L^T (1 / L_jj on its diagonal), K_{t+1}, k_{t+1},
 // L_{t+1} (nullptr skips a store).  Returns true on a failed pivot.
 // Tensor-core stages of input width <= 32: loaded says that A, B, a are in the workspace already, and
 // next() is called once they are no longer needed (it may start the next stage's copies).
@@ -728,7 +713,8 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
             factor_block<T, MT, ld, MHE_TEAM>(s.G, s.K, s.tmp, piv_rel, s.sc + 1);
             wsync();
             const bool bad = s.sc[1] != 0;
-            solve_columns<T, NX, MT, ld, 1>(s.PB, s.PB, s.G, s.K, false, Lgout, Kout, kout, nullptr);
+            if (Lgout) store_factor<T, MT, ld>(Lgout, s.G);
+            solve_columns<T, NX, MT, ld, 1>(s.PB, s.PB, s.G, s.K, false, Kout, kout, nullptr);
             wsync();
             prod<T, NX, NX, MT, ld, ld, true, 0, MHE_TEAM>(
                 s.PB, s.PB, [](int, int) { return None(); }, [&](int i, int j, T v, None) {
@@ -764,12 +750,12 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
         else if (kout)
             wfor(MT, [&](int j) { kout[j] = s.k[j]; });
     }
-    // P -= Y^T Y (symmetric),  Psi = A^T u - l_x + K^T g,  store L^{-T}
+    // P -= Y^T Y (symmetric),  Psi = A^T u - l_x + K^T g,  store L (no barrier: G keeps until the next stage)
     wgemm_tn<T, NX, NX, MT, ld, ld, true>([&](int i, int j) { return s.P[i + j * ld]; }, s.PB, s.PB, (T)-1,
                                           [&](int i, int j, T v) { s.P[i + j * ld] = v; s.P[j + i * ld] = v; });
     wgemm_tn<T, NX, 1, MT, ld, 0>([&](int i, int) { return s.tv[i] - X::lx(st, i); }, s.K, s.g, (T)1,
                                   [&](int i, int, T v) { s.Psi[i] = v; });
-    if (Lgout) store_inverse<T, NX, MT>(s, Lgout);
+    if (Lgout) store_factor<T, MT, ld>(Lgout, s.G);
     if (!want_v) return bad;
     // e = a + B k
     wgemm<T, NX, 1, MT>([&](int i, int) { return s.e[i]; }, [&](int i, int j) { return s.B[i + j * ld]; },

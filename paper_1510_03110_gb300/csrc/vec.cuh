@@ -9,8 +9,10 @@
 // product reads by columns (A^T u, K^T g) get a padded leading dimension, so the lanes'
 // 16-byte loads fall in distinct bank groups; those read by rows stay as they are.
 //
-// The factorisation stores L^{-1} of each pivot block (chol G = L L^T) instead of L, so
-// k = L^{-T} (L^{-1} g) is two short products instead of two serial substitutions.
+// k = G^{-1} g by two substitutions with the stored factor (factor_solve below).  L^{-1} stored instead and applied as
+// two products was faster by up to 8% of a solve, but its error grows with |L^{-1}| |g|, not with |L^{-1} g|: residuals up
+// to 100 times those of substitutions, and an FP32 interior-point loop (256 of nx = nw = 20, leaves of 16) that did not
+// converge in 150 iterations where it now takes 29.
 //
 // Measured against passes that loaded each stage as they came to it (GB300, first full pass): down pass
 // nx = 24, 535k stages, 1.91 -> 1.36 ms (4.8 TB/s); nx = 12, 1.05M stages, 1.10 -> 0.70 ms; nx = 64, 131k stages,
@@ -198,7 +200,7 @@ constexpr int round_to(int n, int v) { return (n + v - 1) / v * v; }
 
 // offsets (elements of T) of a stage's data in a slot; MT = the stage's input width
 template <typename T, int NX, int MT, int KIND>
-struct RhsSlot {   // right-hand-side pass: [A | B], P, [K | L^{-T}], a, l, k
+struct RhsSlot {   // right-hand-side pass: [A | B], P, [K | L], a, l, k
     static constexpr int V = 16 / (int)sizeof(T);
     static constexpr int ldA = pick_ld(NX, vec_of<T>(NX)), ldK = pick_ld(MT, vec_of<T>(MT));
     static constexpr int oA = 0;
@@ -301,11 +303,57 @@ MHE_DEV void sweep(T* ring, int slot, int len, FL&& load, FS&& step)
 
 // ---- right-hand-side pass -----------------------------------------------------
 
+// out = L^{-T} L^{-1} g for the MT x MT lower triangular L (columns LD apart, 1 / L_jj on the diagonal; what lies above
+// it is not used): a warp's lanes hold the entries, each finished one passed on by a shuffle.  Rows (then
+// columns) are scaled by the lane's own reciprocal pivot, so a step of the chain is a shuffle and an FMA.
+template <typename T, int MT, int LD>
+MHE_DEV void factor_solve(const T* L, const T* g, T* out)
+{
+    constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32, R = (MT + CW - 1) / CW;
+    if (MHE_TEAM > CW && lane_id() >= CW) return;
+    const unsigned mask = CW == 32 ? 0xffffffffu : (((1u << CW) - 1u) << ((threadIdx.x & 31) & ~(CW - 1)));
+    T v[R], inv[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = lane_id() + r * CW;
+        inv[r] = i < MT ? L[i + i * LD] : (T)0;
+        v[r] = i < MT ? g[i] * inv[r] : (T)0;
+    }
+#pragma unroll
+    for (int b = 0; b < R; ++b)
+#pragma unroll 8
+        for (int p = b * CW; p < min_int(MT, (b + 1) * CW); ++p) {
+            const T f = __shfl_sync(mask, v[b], p - b * CW, CW);
+#pragma unroll
+            for (int r = b; r < R; ++r) {
+                const int i = lane_id() + r * CW;
+                if (i > p && i < MT) v[r] -= L[i + p * LD] * inv[r] * f;
+            }
+        }
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] *= inv[r];
+#pragma unroll
+    for (int b = R - 1; b >= 0; --b)
+#pragma unroll 8
+        for (int p = min_int(MT, (b + 1) * CW) - 1; p >= b * CW; --p) {
+            const T f = __shfl_sync(mask, v[b], p - b * CW, CW);
+#pragma unroll
+            for (int r = 0; r <= b; ++r) {
+                const int i = lane_id() + r * CW;
+                if (i < p) v[r] -= L[p + i * LD] * inv[r] * f;
+            }
+        }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = lane_id() + r * CW;
+        if (i < MT) out[i] = v[r];
+    }
+}
+
 // Psi_t from Psi_{t+1} (both in s_psi), k_t to kout:
-//   u = Psi - P a,  [t | g] = [A | B]^T u - [0 | l_w],  Psi = t - l_x + K^T g,
-//   y = L^{-1} g,  k = L^{-T} y
+//   u = Psi - P a,  [t | g] = [A | B]^T u - [0 | l_w],  Psi = t - l_x + K^T g,  k = G^{-1} g
 template <typename T, int NX, int MT, int KIND>
-MHE_DEV void rhs_stage(const T* sl, T* s_psi, T* s_u, T* s_tg, T* s_y, T* kout)
+MHE_DEV void rhs_stage(const T* sl, T* s_psi, T* s_u, T* s_tg, T* kout)
 {
     using S = RhsSlot<T, NX, MT, KIND>;
     T* s_g = s_tg + round_to(NX, S::V);
@@ -324,13 +372,9 @@ MHE_DEV void rhs_stage(const T* sl, T* s_psi, T* s_u, T* s_tg, T* s_y, T* kout)
         });
     }
     wsync();
-    each<NX + MT>([&](int i) {   // column i of [K | L^{-T}]
-        const T d = coldot<MT>(sl + S::oK + i * S::ldK, s_g, (T)0);
-        if (i < NX) s_psi[i] = s_tg[i] - sl[S::ol + i] + d;
-        else s_y[i - NX] = d;
-    });
+    each<NX>([&](int i) { s_psi[i] = s_tg[i] - sl[S::ol + i] + coldot<MT>(sl + S::oK + i * S::ldK, s_g, (T)0); });
+    factor_solve<T, MT, S::ldK>(sl + S::oL, s_g, kout);
     wsync();
-    each<MT>([&](int j) { kout[j] = rowdot<MT, S::ldK>(sl + S::oL + j, s_y, (T)0); });
 }
 
 // x <- A x + B (K x + k) + a  (x in s_x)
@@ -401,9 +445,9 @@ MHE_DEV void rhs_chunk(const LevelArgs<T>& a, int ci, T* smem)
             const int t = cd.t0 + cd.len - 1 - i;
             const long long g = cd.g0 + cd.len - 1 - i;
             if (!UPPER && t == 0)
-                rhs_stage<T, NX, NX, KIND_ARRIVAL>(sl, s_psi, s_u, s_tg, s_y, a.kst0 + (long long)b * NX);
+                rhs_stage<T, NX, NX, KIND_ARRIVAL>(sl, s_psi, s_u, s_tg, a.kst0 + (long long)b * NX);
             else
-                rhs_stage<T, NX, MT, KIND>(sl, s_psi, s_u, s_tg, s_y, a.kst + g * MT);
+                rhs_stage<T, NX, MT, KIND>(sl, s_psi, s_u, s_tg, a.kst + g * MT);
         });
     if (!last) {
         // a^: the closed loop from x = 0 over the chunk (Eq. a)
