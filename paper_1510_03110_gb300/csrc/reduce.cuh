@@ -6,7 +6,7 @@
 //   2. W^T P W + Q, whose blocks are F, H and G (symmetric: one triangle);  W^T u
 //   3. G = L L^T, and beside it A^T V
 //   4. per column, in registers: Y = L^{-1} H^T, y = L^{-1} g, Z = L^{-1} BV and from them
-//      K = -L^{-T} Y, k = L^{-T} y, L_t = -L^{-T} Z, straight to global memory, as L itself
+//      K = -L^{-T} Y, k = L^{-T} y, L_t = -L^{-T} Z, straight to global memory, as L's columns scaled by 1 / L_jj
 //   5. P <- F - Y^T Y,  V <- A^T V - Y^T Z,  Q^_w += Z^T Z,
 //      Psi <- A^T u - l_x - Y^T y,  v <- v + V^T a + Z^T y
 // (K^T B^T V = -Y^T Z and V^T (a + B k) = V^T a + Z^T y, so K, k and L_t are only stored.)
@@ -361,17 +361,26 @@ MHE_DEV int chol_pivoted(T* Gm, double rank_rel, T* permv, T* sc)
     return (int)sc[3];
 }
 
-// The factor in G (columns LD apart) to dst, columns MT apart; whatever lies above the diagonal goes with it
+// The factor L in G (columns LD apart, 1 / L_jj on the diagonal) to dst as the vector passes want it, columns MT apart:
+// L D^{-1/2}, D = diag(L_jj^2), below the diagonal and 1 / D_j on it; whatever lies above goes with it
 template <typename T, int MT, int LD>
 MHE_DEV void store_factor(T* dst, const T* G)
 {
     if constexpr (sizeof(T) == 4 && MT % 4 == 0 && LD % 4 == 0) {
         each<MT * MT / 4>([&](int u) {
             const int i = 4 * (u % (MT / 4)), j = u / (MT / 4);
-            st16(dst + 4 * u, ld16g(G + i + j * LD));
+            const float d = G[j + j * LD];
+            float v[4];
+            ld16(G + i + j * LD, v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] *= d;
+            st16(dst + 4 * u, v);
         });
     } else {
-        each<MT * MT>([&](int r) { dst[r] = G[r % MT + (r / MT) * LD]; });
+        each<MT * MT>([&](int r) {
+            const int j = r / MT;
+            dst[r] = G[r % MT + j * LD] * G[j + j * LD];
+        });
     }
 }
 

@@ -657,7 +657,7 @@ MHE_DEV void tc_stage_products_bf16(Ws<float, NX>& s, const StageRef<float>& st,
 
 // One backward stage of Algorithm 4 (or Algorithms 1-2 when want_v is false).
 // On entry s.P = P_{t+1}, s.Psi = Psi_{t+1}, s.V = V_{t+1}, s.v = v_{t+1},
-// s.Qw = partial Q^_w.  Stores P_{t+1}, L of G_{t+1} = L L^T (1 / L_jj on its diagonal), K_{t+1}, k_{t+1},
+// s.Qw = partial Q^_w.  Stores P_{t+1}, the factor of G_{t+1} (store_factor), K_{t+1}, k_{t+1},
 // L_{t+1} (nullptr skips a store).  Returns true on a failed pivot.
 // Tensor-core stages of input width <= 32: loaded says that A, B, a are in the workspace already, and
 // next() is called once they are no longer needed (it may start the next stage's copies).
@@ -750,7 +750,7 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
         else if (kout)
             wfor(MT, [&](int j) { kout[j] = s.k[j]; });
     }
-    // P -= Y^T Y (symmetric),  Psi = A^T u - l_x + K^T g,  store L (no barrier: G keeps until the next stage)
+    // P -= Y^T Y (symmetric),  Psi = A^T u - l_x + K^T g,  store the factor (no barrier: G keeps until the next stage)
     wgemm_tn<T, NX, NX, MT, ld, ld, true>([&](int i, int j) { return s.P[i + j * ld]; }, s.PB, s.PB, (T)-1,
                                           [&](int i, int j, T v) { s.P[i + j * ld] = v; s.P[j + i * ld] = v; });
     wgemm_tn<T, NX, 1, MT, ld, 0>([&](int i, int) { return s.tv[i] - X::lx(st, i); }, s.K, s.g, (T)1,

@@ -200,7 +200,7 @@ constexpr int round_to(int n, int v) { return (n + v - 1) / v * v; }
 
 // offsets (elements of T) of a stage's data in a slot; MT = the stage's input width
 template <typename T, int NX, int MT, int KIND>
-struct RhsSlot {   // right-hand-side pass: [A | B], P, [K | L], a, l, k
+struct RhsSlot {   // right-hand-side pass: [A | B], P, [K | factor of G], a, l, k
     static constexpr int V = 16 / (int)sizeof(T);
     static constexpr int ldA = pick_ld(NX, vec_of<T>(NX)), ldK = pick_ld(MT, vec_of<T>(MT));
     static constexpr int oA = 0;
@@ -303,21 +303,21 @@ MHE_DEV void sweep(T* ring, int slot, int len, FL&& load, FS&& step)
 
 // ---- right-hand-side pass -----------------------------------------------------
 
-// out = L^{-T} L^{-1} g for the MT x MT lower triangular L (columns LD apart, 1 / L_jj on the diagonal; what lies above
-// it is not used): a warp's lanes hold the entries, each finished one passed on by a shuffle.  Rows (then
-// columns) are scaled by the lane's own reciprocal pivot, so a step of the chain is a shuffle and an FMA.
+// out = G^{-1} g from G = U D U^T: the unit lower triangular U below the diagonal of the MT x MT block at L (columns LD
+// apart), 1 / D_j on it; what lies above is not used.  A warp's lanes hold the entries, each finished one is passed on by
+// a shuffle: with a unit diagonal a step of the chain is a shuffle and an FMA.  (One entry a lane; two at MT = 64.)
 template <typename T, int MT, int LD>
 MHE_DEV void factor_solve(const T* L, const T* g, T* out)
 {
-    constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32, R = (MT + CW - 1) / CW;
+    constexpr int CW = MHE_TEAM < 32 ? MHE_TEAM : 32, R = (MT + CW - 1) / CW, VK = vec_of<T>(MT);
+    static_assert(CW % VK == 0 && LD % VK == 0, "whole vectors of a column");
     if (MHE_TEAM > CW && lane_id() >= CW) return;
     const unsigned mask = CW == 32 ? 0xffffffffu : (((1u << CW) - 1u) << ((threadIdx.x & 31) & ~(CW - 1)));
-    T v[R], inv[R];
+    T v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = lane_id() + r * CW;
-        inv[r] = i < MT ? L[i + i * LD] : (T)0;
-        v[r] = i < MT ? g[i] * inv[r] : (T)0;
+        v[r] = i < MT ? g[i] : (T)0;
     }
 #pragma unroll
     for (int b = 0; b < R; ++b)
@@ -327,20 +327,30 @@ MHE_DEV void factor_solve(const T* L, const T* g, T* out)
 #pragma unroll
             for (int r = b; r < R; ++r) {
                 const int i = lane_id() + r * CW;
-                if (i > p && i < MT) v[r] -= L[i + p * LD] * inv[r] * f;
+                if (i > p && i < MT) v[r] -= L[i + p * LD] * f;
             }
         }
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] *= inv[r];
+    for (int r = 0; r < R; ++r) {
+        const int i = lane_id() + r * CW;
+        if (i < MT) v[r] *= L[i + i * LD];
+    }
 #pragma unroll
     for (int b = R - 1; b >= 0; --b)
-#pragma unroll 8
-        for (int p = min_int(MT, (b + 1) * CW) - 1; p >= b * CW; --p) {
-            const T f = __shfl_sync(mask, v[b], p - b * CW, CW);
+#pragma unroll 2
+        for (int p0 = min_int(MT, (b + 1) * CW) - VK; p0 >= b * CW; p0 -= VK) {
+            T c[R][VK];
 #pragma unroll
             for (int r = 0; r <= b; ++r) {
                 const int i = lane_id() + r * CW;
-                if (i < p) v[r] -= L[p + i * LD] * inv[r] * f;
+                if (i < MT) ldv(L + i * LD + p0, c[r]);
+            }
+#pragma unroll
+            for (int q = VK - 1; q >= 0; --q) {
+                const T f = __shfl_sync(mask, v[b], p0 + q - b * CW, CW);
+#pragma unroll
+                for (int r = 0; r <= b; ++r)
+                    if (lane_id() + r * CW < p0 + q) v[r] -= c[r][q] * f;
             }
         }
 #pragma unroll
