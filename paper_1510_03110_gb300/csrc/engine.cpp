@@ -705,7 +705,7 @@ constexpr int kPassRounds = 4;   // corrections launched pass by pass before the
 // resume: a larger batch's last corrections.  Its passes are launched one by one for the first kPassRounds
 // corrections; what is left then is usually nothing or a few instances, and the corrections still allowed
 // would cost a dozen launches each: one launch takes them, whose clusters without work return at once.  Where the
-// instances that work on would make that much the slower way (few of them, long horizons: solve_rule.h), the
+// instances that work on would make that much the slower way (very long horizons: solve_rule.h), the
 // passes go on.
 bool Engine::has_fused(bool fp64) const
 {

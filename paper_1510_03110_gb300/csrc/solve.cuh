@@ -290,7 +290,7 @@ int solve_cluster(int fp64, int mhe, int batch, int max_N)
 template <int NX, int NW, int NY>
 int resume_cluster(int fp64, int mhe, int batch, int max_N)
 {
-    return resumed_cluster(NX, solve_room_of<NX, NW, NY>(fp64, mhe), batch, max_N);
+    return resumed_cluster(solve_room_of<NX, NW, NY>(fp64, mhe), batch, max_N);
 }
 
 MHE_TEAM_NS_END

@@ -43,25 +43,39 @@ inline int fused_cluster(int nx, const SolveRoom& r, int batch, int max_N)
     return max_N <= solve_stages(nx) * c * r.teams ? c : 0;
 }
 
-// CTAs per instance of a larger batch's corrections after the first four, in one launch, or 0 to go on with a launch
-// per pass.  A solve that has converged by then (the usual one) saves the empty passes of every correction still
-// allowed; one that has not should not pay much for it, whether one instance works on or all do: one CTA, or two,
-// which is as far as the few chunks of an instance keep the teams busy.  Measured, twelve corrections allowed,
-// passes and clusters of 1, 2, 4, with none, a few and all instances working on after the fourth:
-//   MHE form, 1024 of nx = 6, N <= 2048:  4.11  3.74 3.74 3.75;  7.43  6.76 6.69 6.70;  16.2  19.0 20.7 28.8
-//   MHE form, 200 of nx = 12, N <= 300:   1.03  0.73 0.73 0.73;  1.50  1.23 1.21 1.21;   2.5   3.5  3.7  5.6
-//   Q form, 500 of nx = 4, N <= 512:      1.03  0.65 0.65 0.65;  1.68  1.44 1.38 1.35;   3.0   3.3  4.4  6.5
-//   Q form, 256 of nx = 12, N <= 512:     1.31  0.92 0.92 0.93;  2.48  2.23 2.15 2.11;   4.7   7.5  7.4  9.6
-// Left to the passes: few instances or long horizons (16 corrections used: one of nx = 20, N = 16384, 5.1 by passes
-// and 55 resumed with four CTAs; one of nx = 24, N = 2000 2.8 and 9.6), horizons with fewer chunks than teams (2000
-// of nx = 4, N <= 60: all 1.8 and 3.6), and above nx = 8 large batches (1024 of nx = 12, N <= 512: none 3.1 and
-// 2.8, all 11.2 and 18.9).
-inline int resumed_cluster(int nx, const SolveRoom& r, int batch, int max_N)
+// CTAs per instance of the corrections after the first four, in one launch, or 0 to go on with a launch per pass.  A solve
+// that has converged by then (the usual one) saves the empty passes of every correction still allowed, 0.04 each: 0.5
+// with 16 allowed.  One that has not should not pay much for it, whether one instance works on or all do.  So few
+// instances take clusters that fill the GPU, many take one CTA, more (up to four) where a single instance of the
+// longest horizon would leave a team more than 64 stages; beyond 64 a team (32 with eight CTAs and more, which only few
+// instances take and then leave most of the GPU idle) the passes go on.  Measured (nx, batch, N; passes and this rule's
+// cluster), 16 corrections allowed, converged after four or before, and all 16 used:
+//   24, 1, 1000             1.46  0.94 (16 CTAs);    2.73  3.08    (four CTAs: 5.91)
+//   24, 1, 2000             1.57  1.03 (16);         2.97  4.25    (four: 10.2)
+//   12, 1, 6000             1.45  0.86 (16);         2.94  4.28    (four: 11.0)
+//   24, 8, 1000             1.94  1.34 (8);          3.91  4.84
+//   20, 30, <= 512          1.50  0.98 (4);          3.37  4.61
+//   24, 60, <= 600          2.56  2.04 (2);          5.91  7.95
+//   24, 512, <= 2048        26.9  26.4 (4);          83.5  163     (one CTA: 106)
+//   12, 1024, <= 2048       12.2  11.7 (2);          47.5  80.8    (four: 127)
+//   12, 1024, <= 512        4.75  4.15 (1);          16.0  23.0
+//   6, 1024, <= 2048        5.56  5.01 (1);          20.8  25.3
+//   4, 2000, <= 60          0.97  0.53 (1);          2.21  4.41    (four: 16.2)
+// Left to the passes: 20, 1, 16384 (2.46 and 1.80 converged, but 5.2 and 17.5 with 16 CTAs, 59 with four).
+inline int resumed_cluster(const SolveRoom& r, int batch, int max_N)
 {
-    if (2 * batch < r.sms || max_N < 4 * r.teams || (nx > 8 && batch > 2 * r.sms)) return 0;
-    const int most = (nx <= 8 ? 32 : solve_stages(nx)) * r.teams;   // stages of one CTA
-    if (r.resident[0] > 0 && max_N <= most) return 1;
-    return r.resident[1] > 0 && max_N <= 2 * most ? 2 : 0;
+    const int room = r.sms * 11 / 10;
+    int c = 1, i = 0;
+    if (r.resident[0] < 1) return 0;
+    while (i + 1 < kSolveSizes && batch <= r.resident[i + 1] && batch * c * 2 <= room) {
+        c *= 2;
+        ++i;
+    }
+    while (c < 4 && r.resident[i + 1] > 0 && max_N > 64 * c * r.teams) {
+        c *= 2;
+        ++i;
+    }
+    return max_N <= (c >= 8 ? 32 : 64) * c * r.teams ? c : 0;
 }
 
 }  // namespace mhe

@@ -75,8 +75,9 @@ def test_last_corrections_in_one_launch(n, m, form, tol):
     (6, 3, [2 + (37 * i) % 290 for i in range(180)], True),
     (12, 6, [2 + (37 * i) % 290 for i in range(180)], True),
     (20, 10, [2 + (7 * i) % 60 for i in range(200)], True),
-    (20, 10, [1500], False), (24, 12, [900, 5], False),                 # a long horizon, alone or nearly
-    (12, 6, [2 + (37 * i) % 290 for i in range(320)], False)])          # many instances of longer stages
+    (20, 10, [1500], True), (24, 12, [900, 5], True),                   # a long horizon, alone or nearly
+    (12, 6, [2 + (37 * i) % 290 for i in range(320)], True),            # many instances of longer stages
+    (20, 10, [4500], False), (12, 6, [9000, 3], False)])                # horizons too long for sixteen CTAs
 def test_late_corrections_take_the_route_of_the_rule(n, m, Ns, resumed, form):
     """More than four corrections: the rest in one launch, or pass by pass to the end; equal bits either way."""
     insts = [synth.mhe_instance(4400 + i % 40, n, m, m, N) for i, N in enumerate(Ns)]
