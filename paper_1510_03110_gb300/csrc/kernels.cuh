@@ -484,10 +484,21 @@ ShapeEntry make_shape()
     return e;
 }
 
-// A level's reduction with this unit's wider team.  Up to how many chunks it pays, from both sides measured
-// on GB300: FP64 nx = 20, 512 leaf chunks 2.37 -> 2.04 ms (32 -> 128 lanes), 128 master chunks 0.58 -> 0.22 ms; FP64
-// nx = 12, 316 chunks 0.29 -> 0.14 ms, 1125 chunks 0.36 -> 0.33 ms (16 -> 128 lanes); FP32 nx = 24, 362 chunks 41 -> 33
-// us, 1201 chunks 170 -> 175 us.
+// A level's reduction with this unit's wider team, for levels of few chunks: there the length of one chunk's chain is
+// the time.  The limits are four (eight) chunks for each of the GPU's 152 SMs.  Measured (GB300, a level's reduction, own
+// team and wider one, ratio of the times; leaf levels of 16 stages and master levels of four, 19 to 6080 chunks):
+//             up to 152    304          608          760          912          1216
+//   FP64 n=4  0.70-0.97    0.70-0.97    0.71-0.80    0.71-0.80    0.70-0.80    0.80-1.35
+//   FP64 n=6  0.50-0.74    0.50-0.72    0.51-0.60    0.51-0.59    0.51-0.59    0.89-1.07
+//   FP64 12   0.27-0.40    0.32-0.48    0.54-0.59    0.91-0.92    1.06-1.07    0.87-0.94
+//   FP64 20   0.33-0.47    0.48-0.59    0.87-0.88    1.22-1.31    0.94-1.32    0.76-0.84
+//   FP64 24   0.32-0.44    0.47-0.57    0.68-0.88    0.77-1.30    0.78-0.88    0.73-0.85
+//   FP32 4, 6 0.67-0.89    0.68-0.85    0.66-0.74    0.66-0.71    0.67-0.74    0.67-0.78
+//   FP32 12   0.53-0.88    0.53-0.85    0.58-0.75    1.04-1.23    1.04-1.24    0.92-1.15
+//   FP32 20   0.62-0.81    0.66-0.83    0.82-0.94    1.14-1.21    1.20-1.28    1.25-1.37
+//   FP32 24   0.60-0.73    0.62-0.79    0.70-0.83    1.00-1.03    1.16-1.22    0.74-1.17
+// (nx = nw = 20 as nx = 20.)  Up to 608 the wider team wins for every shape; beyond it depends on how the chunks fill the
+// last wave, and only FP64 nx = 12 keeps it further, where it loses at most 7% and wins 13%.
 template <int NX, int NW>
 WideEntry make_wide()
 {
