@@ -471,13 +471,7 @@ MHE_DEV void tc_stage_products(Ws<float, NX>& s, const StageRef<float>& st, TcSt
                 for (int i = 0; i < 16; ++i) qv[i] = row ? X::q(st, r, c + 16 + i) : 0.f;
             }
             // c is a multiple of 16 and n, n + m are too: a block lies in one of P, H or G
-            if (r < NX && c >= NX && MT <= 32) {   // H^T by columns, where the column solves want it
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float x[4] = {v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]};
-                    st16(s.PB + r * ld + (c - NX) + 4 * q, x);
-                }
-            } else if (r < NX) {
+            if (r < NX) {
                 float* dst = c < NX ? s.P + r + c * ld : s.H + r + (c - NX) * ld;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) dst[i * ld] = v[i];
@@ -635,13 +629,7 @@ MHE_DEV void tc_stage_products_bf16(Ws<float, NX>& s, const StageRef<float>& st,
 #pragma unroll
                 for (int i = 0; i < 16; ++i) qv[i] = row ? X::q(st, r, c + 16 + i) : 0.f;
             }
-            if (r < NX && c >= NX && MT <= 32) {   // H^T by columns, where the column solves want it
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float x[4] = {v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]};
-                    st16(s.PB + r * ld + (c - NX) + 4 * q, x);
-                }
-            } else if (r < NX) {
+            if (r < NX) {
                 float* dst = c < NX ? s.P + r + c * ld : s.H + r + (c - NX) * ld;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) dst[i * ld] = v[i];
@@ -659,20 +647,14 @@ MHE_DEV void tc_stage_products_bf16(Ws<float, NX>& s, const StageRef<float>& st,
 // On entry s.P = P_{t+1}, s.Psi = Psi_{t+1}, s.V = V_{t+1}, s.v = v_{t+1},
 // s.Qw = partial Q^_w.  Stores P_{t+1}, the factor of G_{t+1} (store_factor), K_{t+1}, k_{t+1},
 // L_{t+1} (nullptr skips a store).  Returns true on a failed pivot.
-// Tensor-core stages of input width <= 32: loaded says that A, B, a are in the workspace already, and
-// next() is called once they are no longer needed (it may start the next stage's copies).
-struct NoNext {
-    MHE_DEV void operator()() const {}
-};
-template <typename T, int NX, int MT, int KIND, int TC = 0, class FN = NoNext>
+template <typename T, int NX, int MT, int KIND, int TC = 0>
 MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout, T* Kout,
-                         T* kout, T* Lout, bool want_v, double piv_rel, TcState* tcs = nullptr, bool loaded = false,
-                         FN&& next = FN())
+                         T* kout, T* Lout, bool want_v, double piv_rel, TcState* tcs = nullptr)
 {
     constexpr int ld = Ws<T, NX>::ld;
     using X = Acc<T, KIND, NX, MT>;
     if (Pout) store_block<T, NX, NX, ld>(Pout, s.P, (T)1, 0, [](int) {});
-    if (!loaded) load_AB<T, NX, MT, KIND>(s, st);
+    load_AB<T, NX, MT, KIND>(s, st);
     bool on_tc = false;
     if constexpr (TC != 0) on_tc = !want_v;
     if (on_tc) {
@@ -703,28 +685,6 @@ MHE_DEV bool reduce_step(Ws<T, NX>& s, const StageRef<T>& st, T* Pout, T* Lgout,
                                   [&](int j, int, T v) { s.g[j] = v; });
     wgemm_tn<T, NX, 1, NX, ld, 0>([&](int, int) { return (T)0; }, s.A, s.u, (T)1,
                                   [&](int i, int, T v) { s.tv[i] = v; });
-    if constexpr (TC != 0 && MT <= 32) {
-        if (on_tc) {
-            // [Y | y] by columns in PB (H^T is there) and the column after it, the factor by rows in K: one
-            // column a lane through both substitutions; P -= Y^T Y,  Psi = A^T u - l_x - Y^T y
-            T* y = s.PB + NX * ld;
-            next();
-            each<MT>([&](int j) { y[j] = s.g[j]; });
-            factor_block<T, MT, ld, MHE_TEAM>(s.G, s.K, s.tmp, piv_rel, s.sc + 1);
-            wsync();
-            const bool bad = s.sc[1] != 0;
-            if (Lgout) store_factor<T, MT, ld>(Lgout, s.G);
-            solve_columns<T, NX, MT, ld, 1>(s.PB, s.PB, s.G, s.K, false, Kout, kout, nullptr);
-            wsync();
-            prod<T, NX, NX, MT, ld, ld, true, 0, MHE_TEAM>(
-                s.PB, s.PB, [](int, int) { return None(); }, [&](int i, int j, T v, None) {
-                    s.P[i + j * ld] = s.P[j + i * ld] = (i < j ? s.P[i + j * ld] : s.P[j + i * ld]) - v;
-                });
-            each<NX>([&](int i) { s.Psi[i] = s.tv[i] - X::lx(st, i) - coldot<MT>(s.PB + i * ld, y, (T)0); });
-            wsync();
-            return bad;
-        }
-    }
     const bool bad = chol_G<T, NX, MT>(s, piv_rel);
     // [Y | y] = Lg^{-1} [H^T | g] (Y in PB, y in tmp);  K = -Lg^{-T} Y (s.K),  k = Lg^{-T} y = G^{-1} g (s.k)
     {
@@ -815,7 +775,6 @@ MHE_DEV void reduce_chunk(const LevelArgs<T>& a, int ci, T* smem, TcState* tcs =
         }
     });
     int bad_t = -1;
-    bool loaded = false;   // the stage's A, B, a are on their way into the workspace (tensor-core leaf stages)
     if (!UPPER) prefetch_leaf<T, NX, NW>(a, b, cd.t0 + cd.len - 1);
     for (int tt = cd.len - 1; tt >= 0; --tt) {
         const int t = cd.t0 + tt;
@@ -833,24 +792,10 @@ MHE_DEV void reduce_chunk(const LevelArgs<T>& a, int ci, T* smem, TcState* tcs =
                 a.Lgst0 + (long long)b * NX * NX, a.Kst0 + (long long)b * NX * NX, a.kst0 + (long long)b * NX,
                 last ? nullptr : a.Lst0 + (long long)b * NX * NX, !last, a.piv_rel, tcs);
         } else {
-            if (loaded) {
-                cp_wait<0>();
-                wsync();
-            }
-            const bool here = loaded;
-            loaded = false;
             bad = reduce_step<T, NX, NW, KIND_LEAF, TC>(
                 s, Addr<T, NX, NW>::leaf(a, b, t), a.store_P ? a.Pst + g * NX * NX : nullptr,
                 a.Lgst + g * NW * NW, a.Kst + g * NW * NX, a.kst + g * NW,
-                last ? nullptr : a.Lst + g * NW * NX, !last, a.piv_rel, tcs, here, [&] {
-                    if (tt == 0 || t < 2) return;
-                    const StageRef<T> nx = Addr<T, NX, NW>::leaf(a, b, t - 1);
-                    async_block<T, NX, NX, ld>(s.A, nx.A);
-                    async_block<T, NX, NW, ld>(s.B, nx.B);
-                    async_vec<T, NX>(s.e, nx.a);
-                    cp_commit();
-                    loaded = true;
-                });
+                last ? nullptr : a.Lst + g * NW * NX, !last, a.piv_rel, tcs);
         }
         if (bad && bad_t < 0) bad_t = t;
     }
