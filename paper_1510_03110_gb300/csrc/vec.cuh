@@ -16,7 +16,7 @@
 //
 // Measured against passes that loaded each stage as they came to it (GB300, first full pass): down pass
 // nx = 24, 535k stages, 1.91 -> 1.36 ms (4.8 TB/s); nx = 12, 1.05M stages, 1.10 -> 0.70 ms; nx = 64, 131k stages,
-// 3.57 -> 1.59 ms; right-hand-side pass nx = 24 1.45 -> 1.09 ms, nx = 64 3.11 -> 1.04 ms; one master level of
+// 3.57 -> 1.59 ms; right-hand-side pass nx = 24 1.45 -> 1.15 ms, nx = 64 3.11 -> 1.39 ms; one master level of
 // four-stage chunks at nx = 24 22 -> 14 us.
 #pragma once
 #include <stdint.h>
