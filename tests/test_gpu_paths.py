@@ -105,6 +105,22 @@ def test_levels_of_many_chunks(n, m, prec, tol):
         assert rel_err(sols[b], ref) <= tol, (b, Ns[b])
 
 
+@pytest.mark.parametrize("n,m", [(6, 3), (12, 6)])
+def test_master_levels_of_many_chunks(n, m):
+    """More chunks than the wider teams take (1216) at a master level too, FP64: the shape's own team, against the oracle."""
+    Ns = [34] * 640
+    insts = [synth.mhe_instance(4600 + i % 64, n, m, m, N) for i, N in enumerate(Ns)]
+    d = device_inputs(insts)
+    s = mhe.Solver(n, m, Ns, prec=mhe.MHE_FP64, leaf_len=8, branching=2, top_len=2)
+    assert mhe.mhe_plan_info(s.ctx)[1][1] > 1216
+    s.close()
+    out, info, _ = _run(d, "solve", mhe.MHE_FP64, False, leaf_len=8, branching=2, top_len=2)
+    assert np.all(info["status"] == 0)
+    sols = split(*out, Ns, n, m)
+    for b in (0, 1, 63, 317, 639):
+        assert rel_err(sols[b], oracle.riccati(oracle.mhe_to_uftoc(insts[b]))) <= 1e-10, b
+
+
 def test_preparation_of_zeros_and_extreme_entries():
     """Entries that leave the fast conversion (zeros, tiny and huge magnitudes) against the FP64 solution."""
     n, m = 6, 3
